@@ -467,6 +467,7 @@ int pa_init(const pa_config* cfg, void* ws, size_t bytes, void* stream, pa_run**
     d.cap_alloc = (uint32_t)l.cap;
     d.R0 = (uint32_t)cfg->R0;
     d.tiles = (uint32_t)l.tiles;
+    d.slice_lg = pa::resample_slices((uint64_t)l.tiles);
     d.mn_cum = l.mn_cum ? (unsigned long long*)(base + l.mn_cum) : nullptr;
     d.mn_tiles = l.mn_tiles ? (unsigned long long*)(base + l.mn_tiles) : nullptr;
     r->hist_bytes = 16 + (size_t)l.bins * 4;
@@ -1320,6 +1321,7 @@ int batch_init(pa_run* const* runs, int32_t nruns, const int32_t* steps_left, vo
     for (double& m : b->prof_ms) m = 0.0;
     std::vector<pa::RunDev> h_runs;
     std::vector<uint32_t> tile_base(1, 0u);
+    uint64_t tiles = 0;
     for (int32_t i = 0; i < nruns; ++i) {
         pa_run* r = runs[i];
         if (!r || r->gather_pending) {
@@ -1349,7 +1351,13 @@ int batch_init(pa_run* const* runs, int32_t nruns, const int32_t* steps_left, vo
         if (left < b->steps_left) b->steps_left = left;
         b->runs.push_back(r);
         h_runs.push_back(r->d);
-        tile_base.push_back(tile_base.back() + r->d.tiles);
+        tiles += r->d.tiles;
+    }
+    // one launch resamples all runs: slices by the tiles of the whole batch
+    const uint32_t slice_lg = pa::resample_slices(tiles);
+    for (auto& d : h_runs) {
+        d.slice_lg = slice_lg;
+        tile_base.push_back(tile_base.back() + (d.tiles << slice_lg));
     }
     // classes: one sweep kernel instantiation per (layout, dim, L, model)
     for (int32_t i = 0; i < nruns; ++i) {
@@ -1412,6 +1420,7 @@ int batch_init(pa_run* const* runs, int32_t nruns, const int32_t* steps_left, vo
     b->bd.nruns = (uint32_t)nruns;
     b->bd.tile_base = d_tile_base;
     b->bd.total_tiles = tile_base.back();
+    b->bd.slice_lg = slice_lg;
     b->bd.any_poisson = 0;
     b->bd.any_multinomial = 0;
     for (const auto& h : h_runs) {

@@ -88,6 +88,7 @@ struct RunDev {
     uint32_t cap_alloc;         // slots in each buffer
     uint32_t R0;
     uint32_t tiles;             // descriptors available
+    uint32_t slice_lg;          // log2 of the CTAs that share a resample tile (resample_slices)
     uint32_t rk0[10], rk1[10];  // Philox round keys of `seed` (key + r * Weyl constant)
     uint32_t one;               // the value 1, opaque to the compiler (multiply-add tests)
     int32_t theta;              // sweeps per annealing step
@@ -108,8 +109,9 @@ struct RunDev {
 struct BatchDev {
     const RunDev* runs;          // [nruns]
     uint32_t nruns;
-    const uint32_t* tile_base;   // [nruns + 1] prefix sums of each run's resample tiles
-    uint32_t total_tiles;
+    const uint32_t* tile_base;   // [nruns + 1] prefix sums of each run's slices of tiles
+    uint32_t total_tiles;        // slices of all tiles
+    uint32_t slice_lg;           // log2 of the slices of a tile (every run's RunDev::slice_lg)
     uint32_t any_poisson;        // some run resamples by the Poisson rule
     uint32_t any_multinomial;    // some run resamples by multinomial draws
     uint32_t* counters;          // [0]: resample tiles, [1 + c]: sweep chunks of class c
@@ -171,6 +173,82 @@ __device__ __forceinline__ uint32_t pick(const uint4& v, uint32_t j) {
     return j == 0 ? v.x : j == 1 ? v.y : j == 2 ? v.z : v.w;
 }
 
+// Descriptors of a single-pass scan: flag (aggregate or prefix) << 62 | epoch
+// << 32 | value.
+constexpr unsigned long long DESC_AGG = 1ull;
+constexpr unsigned long long DESC_PREFIX = 2ull;
+constexpr unsigned LOOKBACK_SPIN_LIMIT = 1u << 22;
+
+__device__ __forceinline__ void st_release(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ unsigned long long desc_make(unsigned long long flag, uint32_t epoch,
+                                                         uint32_t value) {
+    return (flag << 62) | ((unsigned long long)(epoch & 0x3fffffffu) << 32) | value;
+}
+
+// Decoupled lookback of tile `tile` > 0, by all NW warps of a CTA: the sum of
+// the counts of all tiles before it.  Warp w watches the 32 predecessors tile -
+// 1 - 32 w - lane; as soon as a prefix is among them and every nearer one has
+// published its aggregate the warp's sum is known, without a prefix when all
+// 32 aggregates are there, and the CTA's window of 32 NW tiles moves on.  The
+// wait is a chain of L2 round trips (about 0.7 us each), as long as the number
+// of windows between a tile and the nearest prefix.  Bounded:
+// after LOOKBACK_SPIN_LIMIT polls without progress it returns what it has and
+// ok = false.  All threads return the same values; sm is free for reuse only
+// after a further barrier.
+template <int NW>
+struct LookSmem {
+    uint32_t sum[2][NW], found[2][NW];
+};
+template <int NW>
+__device__ __forceinline__ uint32_t lookback(const unsigned long long* desc, uint32_t tile,
+                                             uint32_t epoch, LookSmem<NW>& sm, bool& ok) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t tag = epoch & 0x3fffffffu;
+    uint32_t excl = 0;
+    ok = true;
+    int ph = 0;
+    for (int64_t top = (int64_t)tile - 1;; top -= 32 * NW, ph ^= 1) {
+        const int64_t p = top - 32 * wid - lane;
+        unsigned spins = 0;
+        for (;;) {
+            unsigned long long v = desc_make(DESC_PREFIX, epoch, 0);  // before tile 0: nothing
+            if (p >= 0) v = ld_acquire(desc + p);
+            const bool ready = (v >> 62) != 0 && ((uint32_t)(v >> 32) & 0x3fffffffu) == tag;
+            const unsigned have = __ballot_sync(0xffffffffu, ready);
+            const unsigned pref = __ballot_sync(0xffffffffu, ready && (v >> 62) == DESC_PREFIX);
+            // the lanes up to the nearest prefix are needed, all of them without one
+            const unsigned need = pref ? (pref ^ (pref - 1u)) : 0xffffffffu;
+            const bool late = (have & need) != need;
+            if (!late || ++spins >= LOOKBACK_SPIN_LIMIT) {
+                const uint32_t sum =
+                    __reduce_add_sync(0xffffffffu, (need & have) >> lane & 1u ? (uint32_t)v : 0u);
+                if (lane == 0) {
+                    sm.sum[ph][wid] = sum;
+                    sm.found[ph][wid] = late ? 2u : pref ? 1u : 0u;
+                }
+                break;
+            }
+            if (spins > 64) __nanosleep(64);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            excl += sm.sum[ph][w];
+            if (sm.found[ph][w] == 2u) ok = false;
+            if (sm.found[ph][w]) return excl;
+        }
+    }
+}
+
 // ---- launchers (defined in the kernel translation units) ----------------
 bool sweep_supported(int layout, int dim, int L);
 cudaError_t launch_init(const RunDev& d, cudaStream_t s);
@@ -223,5 +301,18 @@ int l64_batched_grid(const RunDev& proto);
 constexpr int RS_THREADS = 256;
 constexpr int RS_ITEMS = PA_RS_ITEMS;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
+// log2 of the slices of a tile for `tiles` tiles that one launch resamples.
+// One CTA gathers at about 30 GB/s whatever else runs, so the launch needs as
+// many CTAs as the GPU holds (152 x 4); a population of fewer tiles has
+// several CTAs count the whole of a tile (a microsecond or two) and each
+// gather its slice, of at least 32 replicas.
+#ifndef PA_RS_SPREAD
+#define PA_RS_SPREAD 608
+#endif
+inline uint32_t resample_slices(uint64_t tiles) {
+    uint32_t lg = 0;
+    while ((RS_TILE >> (lg + 1)) >= 32 && (tiles << (lg + 1)) <= PA_RS_SPREAD) ++lg;
+    return lg;
+}
 
 }  // namespace pa

@@ -9,7 +9,7 @@
 //              (Eq. 4, renormalised to R0), kept as n_k = floor(tau_k),
 //              F_k = floor(frac(tau_k) 2^32).
 //  k_resample  one pass over the population, one tile of RS_TILE replicas per
-//              CTA: copy counts r_j = n_k + [u_j < F_k] (nearest-integer rule),
+//              CTA (or per group of CTAs that share its gather): copy counts r_j = n_k + [u_j < F_k] (nearest-integer rule),
 //              a single-pass exclusive scan with decoupled lookback across
 //              tiles, and the gather of r_j exact copies of replica j into slots
 //              o_j .. o_j + r_j - 1 of the other population buffer.
@@ -23,25 +23,6 @@
 
 namespace pa {
 namespace {
-
-constexpr unsigned long long DESC_AGG = 1ull;
-constexpr unsigned long long DESC_PREFIX = 2ull;
-constexpr unsigned LOOKBACK_SPIN_LIMIT = 1u << 22;
-
-__device__ __forceinline__ void st_release(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ unsigned long long desc_make(unsigned long long flag, uint32_t epoch,
-                                                         uint32_t value) {
-    return (flag << 62) | ((unsigned long long)(epoch & 0x3fffffffu) << 32) | value;
-}
 
 // The batched kernels stage a run's descriptor in shared memory (PA_RS_STAGE
 // = 1): read from global memory, its fields could alias the kernel's own
@@ -190,30 +171,25 @@ __global__ void __launch_bounds__(256) k_tau_batched(BatchDev b) {
     if (threadIdx.x < 2) d.accum[threadIdx.x] = 0ull;
 }
 
-// PA_RS_COMPACT = 1: the gather walks only the tile's surviving replicas
-// (count > 0), listed in order in shared memory, so that every 16-byte item a
-// thread takes has a load behind it; 0 walks every replica of the tile.
-#ifndef PA_RS_COMPACT
-#define PA_RS_COMPACT 1
-#endif
-
+// The gather walks only the tile's surviving replicas (count > 0), listed in
+// order, so that every 16-byte item a thread takes has a load behind it.
 struct ResampleSmem {
-    uint32_t r[RS_TILE];
-    uint32_t o[RS_TILE];
-#if PA_RS_COMPACT
-    uint32_t surv[RS_TILE];             // tile indices of the surviving replicas
-    uint32_t warp_nz[RS_THREADS / 32];  // survivors before each warp
-    uint32_t nsurv;
-#endif
+    // survivor j of this CTA's slice: tile index, count, first slot
+    uint32_t surv[RS_TILE], r[RS_TILE], o[RS_TILE];
+    uint32_t warp_nz[RS_THREADS / 32];  // survivors of each warp
     uint32_t warp[RS_THREADS / 32];
-    uint32_t tile, excl;
+    uint32_t tile;
+    LookSmem<RS_THREADS / 32> look;
 };
 
-// 16-byte loads in flight per thread in the gather.  Measured on GB300 at 2^21
-// replicas, L = 64 (one-kernel form, same bits): 4 -> 0.368 ms, 5 -> 0.361
-// ms, 6 -> 0.361 ms, 8 with 3 CTAs per SM -> 0.400 ms.
+// 16-byte loads in flight per thread in the gather, within the 64 registers of
+// four CTAs per SM (only the data stays in registers between the loads and the
+// stores).  Measured on GB300, us per launch: 2^21 replicas of 512 bytes 346 (4),
+// 347 (6), 348 (8; 12 at 3 CTAs per SM 365; 4 at 5 CTAs 367); 24 spin-glass runs
+// of 2^15..2^16 in one launch 112 (4), 117 (6), 122 (8).  346 us are 6.1 TB/s over the
+// exact bytes, 0.90 of the measured copy peak: HBM bounds it.
 #ifndef PA_RS_GU
-#define PA_RS_GU 6
+#define PA_RS_GU 4
 #endif
 
 // Counts, scan and gather of tile `tile` of one run (all threads of the CTA).
@@ -253,10 +229,48 @@ __device__ __noinline__ uint32_t poisson_count(const RunDev& d, uint32_t i, uint
     return count;
 }
 
+// Poisson copy counts, one replica per thread: a draw is two or three Philox
+// blocks and a table walk one after the other, so they run over the whole GPU
+// ahead of the scan instead of eight after another in a tile's threads.  The
+// Poisson resample of 2^21 replicas (L = 64) takes 333 us with it on GB300 against
+// 407 with the draws inside the scan kernel, at 89 registers.
+__device__ __forceinline__ void poisson_counts(const RunDev& d, uint32_t first, uint32_t stride,
+                                               uint32_t end) {
+    const uint32_t step = d.st->step;
+    const uint32_t* eb = d.ebin[d.st->src];
+    for (uint32_t i = first; i < end; i += stride) {
+        const uint32_t k = eb[i];
+        d.counts[i] = poisson_count(d, i, step, d.tab_n[k], d.tab_F[k]);
+    }
+}
+
+__global__ void __launch_bounds__(256) k_poisson_counts(__grid_constant__ const RunDev d) {
+    if (!d.st->active) return;
+    poisson_counts(d, blockIdx.x * 256u + threadIdx.x, gridDim.x * 256u, d.st->R_prev);
+}
+
+// Batched: CTA g takes resample tile g of the batch, if its run is on the rule.
+__global__ void __launch_bounds__(RS_THREADS) k_poisson_counts_batched(BatchDev b) {
+    __shared__ RunDev s_d;
+    const uint32_t g = blockIdx.x << b.slice_lg;
+    uint32_t lo = 0, hi = b.nruns;  // tile_base[lo] <= g < tile_base[hi]
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (b.tile_base[mid] <= g) lo = mid;
+        else hi = mid;
+    }
+    if (b.runs[lo].resample != PA_RESAMPLE_POISSON || !b.runs[lo].st->active) return;
+    stage_run(&b.runs[lo], s_d);
+    __syncthreads();
+    const uint32_t base = ((g - b.tile_base[lo]) >> b.slice_lg) * (uint32_t)RS_TILE;
+    const uint32_t R = s_d.st->R_prev;
+    if (base < R)
+        poisson_counts(s_d, base + threadIdx.x, RS_THREADS, min(R, base + (uint32_t)RS_TILE));
+}
+
 // RULE 0 compiles the nearest-integer rule alone (the register budget of the
-// HBM-bound default path); 1 adds the per-run Poisson branch; 2 takes the
-// counts that the multinomial draw has left in d.counts; 3 chooses among the
-// three per run (batches that mix the rules).
+// HBM-bound default path); 2 takes the counts that the Poisson or multinomial
+// draws have left in d.counts; 3 chooses between the two per run (batches).
 //
 // SPLIT = false: the tile also gathers its replicas' spins (the batched form).
 // SPLIT = true: the tile writes, for each slot it fills, the index of the
@@ -264,41 +278,30 @@ __device__ __noinline__ uint32_t poisson_count(const RunDev& d, uint32_t i, uint
 // k_gather copies the spins afterwards over the whole new population (the
 // plain form).
 template <int RULE, bool SPLIT = false>
-__device__ __forceinline__ void resample_tile(const RunDev& d, uint32_t tile, ResampleSmem& sm) {
+__device__ __forceinline__ void resample_tile(const RunDev& d, uint32_t tile, uint32_t slice,
+                                              ResampleSmem& sm) {
     DevState* st = d.st;
-    uint32_t* s_r = sm.r;
-    uint32_t* s_o = sm.o;
     uint32_t* s_warp = sm.warp;
-    uint32_t& s_excl = sm.excl;
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const uint32_t R = st->R_prev, epoch = st->epoch, src = st->src, step = st->step;
     const uint32_t base = tile * RS_TILE;
-    if (base >= R) return;
-    const uint32_t n_in = min((uint32_t)RS_TILE, R - base);
-
+    // every CTA of a tile counts all of it; this one keeps slice [lo, hi)
+    const uint32_t width = (uint32_t)RS_TILE >> d.slice_lg;
+    const uint32_t lo = base + slice * width;
+    if (lo >= R) return;
+    const uint32_t end = min(R, base + (uint32_t)RS_TILE), hi = min(R, lo + width);
     // copy counts, RS_ITEMS consecutive replicas per thread
     const uint32_t* eb = d.ebin[src];
     const uint32_t ctr3 = (TAG_RESAMPLE << 28) | d.instance;
     const uint32_t k0 = (uint32_t)d.seed, k1 = (uint32_t)(d.seed >> 32);
     uint32_t r[RS_ITEMS];
     uint32_t sum = 0;
-    if (RULE == 2 || (RULE == 3 && d.resample == PA_RESAMPLE_MULTINOMIAL)) {
+    const bool drawn = RULE == 2 || (RULE == 3 && d.resample != PA_RESAMPLE_NEAREST);
+    if (drawn) {
 #pragma unroll
         for (int j = 0; j < RS_ITEMS; ++j) {
             const uint32_t i = base + (uint32_t)t * RS_ITEMS + j;
-            const uint32_t v = i < R ? d.counts[i] : 0u;
-            r[j] = v;
-            sum += v;
-        }
-    } else if ((RULE == 1 || RULE == 3) && d.resample == PA_RESAMPLE_POISSON) {
-#pragma unroll
-        for (int j = 0; j < RS_ITEMS; ++j) {
-            const uint32_t i = base + (uint32_t)t * RS_ITEMS + j;
-            uint32_t v = 0;
-            if (i < R) {
-                const uint32_t k = eb[i];
-                v = poisson_count(d, i, step, d.tab_n[k], d.tab_F[k]);
-            }
+            const uint32_t v = i < end ? d.counts[i] : 0u;
             r[j] = v;
             sum += v;
         }
@@ -307,19 +310,29 @@ __device__ __forceinline__ void resample_tile(const RunDev& d, uint32_t tile, Re
     for (int j0 = 0; j0 < RS_ITEMS; j0 += 4) {
         const uint32_t i0 = base + (uint32_t)t * RS_ITEMS + j0;
         uint4 u = make_uint4(0, 0, 0, 0);
-        if (i0 < R) u = philox(i0 >> 2, step, 0u, ctr3, k0, k1);
+        uint32_t lev[4] = {0, 0, 0, 0};
+        if (i0 < end) u = philox(i0 >> 2, step, 0u, ctr3, k0, k1);
+        if (i0 + 4 <= end) {  // i0 is a multiple of 4: one 16-byte load
+            const uint4 e4 = *reinterpret_cast<const uint4*>(eb + i0);
+            lev[0] = e4.x, lev[1] = e4.y, lev[2] = e4.z, lev[3] = e4.w;
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (i0 + j < end) lev[j] = eb[i0 + j];
+        }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const uint32_t i = i0 + j;
             uint32_t v = 0;
-            if (i < R) {
-                const uint32_t k = eb[i];
+            if (i0 + j < end) {
+                const uint32_t k = lev[j];
                 v = d.tab_n[k] + (pick(u, (uint32_t)j) < d.tab_F[k] ? 1u : 0u);
             }
             r[j0 + j] = v;
             sum += v;
         }
     }
+    const uint32_t i_first = base + (uint32_t)t * RS_ITEMS;
+    const bool mine = i_first >= lo && i_first < hi;  // a slice holds whole threads
     // block-wide exclusive scan of the per-thread sums
     uint32_t incl = sum;
 #pragma unroll
@@ -328,11 +341,11 @@ __device__ __forceinline__ void resample_tile(const RunDev& d, uint32_t tile, Re
         if (lane >= o) incl += y;
     }
     if (lane == 31) s_warp[wid] = incl;
-#if PA_RS_COMPACT
     // and of the per-thread survivor counts
     uint32_t nz = 0;
 #pragma unroll
     for (int j = 0; j < RS_ITEMS; ++j) nz += r[j] ? 1u : 0u;
+    if (!mine) nz = 0;
     uint32_t nzi = nz;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -340,159 +353,123 @@ __device__ __forceinline__ void resample_tile(const RunDev& d, uint32_t tile, Re
         if (lane >= o) nzi += y;
     }
     if (lane == 31) sm.warp_nz[wid] = nzi;
-#endif
     __syncthreads();
-#if PA_RS_COMPACT
-    if (wid == 1) {
-        const uint32_t w = lane < RS_THREADS / 32 ? sm.warp_nz[lane] : 0u;
-        uint32_t wi = w;
+    uint32_t before = 0, total = 0;  // counts of the warps before this one, of the tile
+    uint32_t before_nz = 0, nsurv = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += y;
-        }
-        if (lane < RS_THREADS / 32) sm.warp_nz[lane] = wi - w;
-        if (lane == RS_THREADS / 32 - 1) sm.nsurv = wi;
+    for (int w = 0; w < RS_THREADS / 32; ++w) {
+        if (w == wid) before = total;
+        total += s_warp[w];
+        if (w == wid) before_nz = nsurv;
+        nsurv += sm.warp_nz[w];
     }
-#endif
-    if (wid == 0) {
-        uint32_t w = lane < RS_THREADS / 32 ? s_warp[lane] : 0u;
-        uint32_t wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += y;
+    uint32_t excl = 0;
+    if (tile == 0) {
+        // the test hook withholds tile 0's prefix, so that the bounded waits of
+        // the tiles after it run out (PA_DEBUG_WITHHOLD_PREFIX)
+        if (t == 0 && slice == 0 && !(d.debug & PA_DEBUG_WITHHOLD_PREFIX))
+            st_release(&d.desc[0], desc_make(DESC_PREFIX, epoch, total));
+    } else {
+        // slice 0 speaks for the tile: it is claimed first
+        if (t == 0 && slice == 0) st_release(&d.desc[tile], desc_make(DESC_AGG, epoch, total));
+        bool ok;
+        excl = lookback(d.desc, tile, epoch, sm.look, ok);
+        if (t == 0) {
+            if (!ok) atomicOr(&st->status, ST_TIMEOUT);
+            if (slice == 0) st_release(&d.desc[tile], desc_make(DESC_PREFIX, epoch, excl + total));
         }
-        if (lane < RS_THREADS / 32) s_warp[lane] = wi - w;  // exclusive warp offsets
-        const uint32_t total = __shfl_sync(0xffffffffu, wi, RS_THREADS / 32 - 1);
-        // decoupled lookback across tiles (one thread)
-        if (lane == 0) {
-            uint32_t excl = 0;
-            if (tile == 0) {
-                // the test hook withholds tile 0's prefix, so that tile 1's
-                // bounded wait runs out (PA_DEBUG_WITHHOLD_PREFIX)
-                if (!(d.debug & PA_DEBUG_WITHHOLD_PREFIX))
-                    st_release(&d.desc[0], desc_make(DESC_PREFIX, epoch, total));
-            } else {
-                st_release(&d.desc[tile], desc_make(DESC_AGG, epoch, total));
-                int p = (int)tile - 1;
-                for (;;) {
-                    unsigned long long v = 0;
-                    unsigned spins = 0;
-                    bool ok = false;
-                    for (;;) {
-                        v = ld_acquire(&d.desc[p]);
-                        if ((v >> 62) != 0 && ((v >> 32) & 0x3fffffffu) == (epoch & 0x3fffffffu)) {
-                            ok = true;
-                            break;
-                        }
-                        if (++spins >= LOOKBACK_SPIN_LIMIT) break;
-                        if (spins > 64) __nanosleep(64);
-                    }
-                    if (!ok) {
-                        atomicOr(&st->status, ST_TIMEOUT);
-                        break;
-                    }
-                    excl += (uint32_t)(v & 0xffffffffu);
-                    if ((v >> 62) == DESC_PREFIX || p == 0) break;
-                    --p;
+    }
+    uint32_t o = excl + before + (incl - sum);
+    uint32_t p = before_nz + (nzi - nz);
+    if (mine)
+#pragma unroll
+    for (int j0 = 0; j0 < RS_ITEMS; j0 += 4) {
+        const uint32_t li0 = (uint32_t)t * RS_ITEMS + j0;
+        const uint32_t i0 = base + li0;
+        uint32_t oo[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            oo[j] = o;
+            o += r[j0 + j];
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (r[j0 + j]) {  // 0 beyond R
+                sm.surv[p] = li0 + j;
+                sm.r[p] = r[j0 + j];
+                sm.o[p++] = oo[j];
+            }
+        }
+        if (i0 + 4 <= end) {  // i0 is a multiple of 4: 16-byte stores
+            const uint4 r4 = make_uint4(r[j0], r[j0 + 1], r[j0 + 2], r[j0 + 3]);
+            const uint4 o4 = make_uint4(oo[0], oo[1], oo[2], oo[3]);
+            if (!drawn) *reinterpret_cast<uint4*>(d.counts + i0) = r4;
+            *reinterpret_cast<uint4*>(d.offsets + i0) = o4;
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (i0 + j < end) {
+                    if (!drawn) d.counts[i0 + j] = r[j0 + j];
+                    d.offsets[i0 + j] = oo[j];
                 }
-                st_release(&d.desc[tile], desc_make(DESC_PREFIX, epoch, excl + total));
             }
-            s_excl = excl;
+        }
+        if (i0 < R && R - 1 - i0 < 4) {  // the population's last replica
+            if (o > d.cap) atomicOr(&st->status, ST_CAPACITY);
+            if (o == 0) atomicOr(&st->status, ST_EMPTY);
+            st->R = o > d.cap ? d.cap : o;
         }
     }
     __syncthreads();
-    uint32_t o = s_excl + s_warp[wid] + (incl - sum);
-#if PA_RS_COMPACT
-    uint32_t p = sm.warp_nz[wid] + (nzi - nz);
-#endif
-#pragma unroll
-    for (int j = 0; j < RS_ITEMS; ++j) {
-        const uint32_t li = (uint32_t)t * RS_ITEMS + j;
-        const uint32_t i = base + li;
-#if PA_RS_COMPACT
-        if (r[j]) sm.surv[p++] = li;  // r[j] = 0 beyond R
-#endif
-        if (i < R) {
-            s_r[li] = r[j];
-            s_o[li] = o;
-            d.counts[i] = r[j];
-            d.offsets[i] = o;
-            if (i == R - 1) {
-                const uint32_t Rnew = o + r[j];
-                if (Rnew > d.cap) atomicOr(&st->status, ST_CAPACITY);
-                if (Rnew == 0) atomicOr(&st->status, ST_EMPTY);
-                st->R = Rnew > d.cap ? d.cap : Rnew;
-            }
-        }
-        o += r[j];
-    }
-    __syncthreads();
-#if PA_RS_COMPACT
-    if (t == 0) atomicAdd(&st->sources, (unsigned long long)sm.nsurv);
-#endif
+    if (t == 0) atomicAdd(&st->sources, (unsigned long long)nsurv);
 
-#if PA_RS_COMPACT
-    const uint32_t nlist = sm.nsurv;  // gather item j of the list: replica surv[j]
-#else
-    const uint32_t nlist = n_in;
-#endif
     // gather: 16-byte chunks, consecutive threads on consecutive chunks; GU
-    // independent loads in flight per thread before their stores
+    // independent loads in flight per thread before their stores, whose
+    // survivor is looked up again (shared memory) rather than kept in registers
     if (!SPLIT) {
-    constexpr int GU = PA_RS_GU;
-    const uint32_t CH = d.stride >> 4;
-    const uint4* __restrict__ srcp = reinterpret_cast<const uint4*>(d.spins[src]) + (size_t)base * CH;
-    uint4* __restrict__ dstp = reinterpret_cast<uint4*>(d.spins[src ^ 1u]);
-    const uint32_t items = nlist * CH;
-    const bool pow2 = (CH & (CH - 1)) == 0;
-    const int shift = __ffs(CH) - 1;
-    for (uint32_t it0 = t; it0 < items; it0 += RS_THREADS * GU) {
-        uint4 v[GU];
-        uint32_t rr[GU], d0[GU], cc[GU];
+        constexpr int GU = PA_RS_GU;
+        const uint32_t CH = d.stride >> 4;
+        // it / CH for it < RS_TILE * CH: the product with ceil(2^32 / CH) is exact
+        // while it * CH < 2^32 (CH <= 1024)
+        const uint32_t recip = CH > 1 ? 0xffffffffu / CH + 1u : 0u;
+        const uint4* __restrict__ srcp =
+            reinterpret_cast<const uint4*>(d.spins[src]) + (size_t)base * CH;
+        uint4* __restrict__ dstp = reinterpret_cast<uint4*>(d.spins[src ^ 1u]);
+        const uint32_t items = nsurv * CH;
+        for (uint32_t it0 = t; it0 < items; it0 += RS_THREADS * GU) {
+            uint4 v[GU];
 #pragma unroll
-        for (int u = 0; u < GU; ++u) {
-            const uint32_t it = it0 + (uint32_t)u * RS_THREADS;
-            rr[u] = 0;
-            if (it < items) {
-                const uint32_t jl = pow2 ? (it >> shift) : (it / CH);
-                cc[u] = it - jl * CH;
-#if PA_RS_COMPACT
-                const uint32_t li = sm.surv[jl];
-#else
-                const uint32_t li = jl;
-#endif
-                rr[u] = s_r[li];
-                d0[u] = s_o[li];
-                if (rr[u]) v[u] = __ldg(srcp + (size_t)li * CH + cc[u]);
+            for (int u = 0; u < GU; ++u) {
+                const uint32_t it = it0 + (uint32_t)u * RS_THREADS;
+                if (it < items) {
+                    const uint32_t jl = recip ? __umulhi(it, recip) : it;
+                    v[u] = __ldg(srcp + (size_t)sm.surv[jl] * CH + (it - jl * CH));
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < GU; ++u) {
+                const uint32_t it = it0 + (uint32_t)u * RS_THREADS;
+                if (it < items) {
+                    const uint32_t jl = recip ? __umulhi(it, recip) : it;
+                    const uint32_t rr = sm.r[jl], d0 = sm.o[jl], c = it - jl * CH;
+                    for (uint32_t k = 0; k < rr; ++k) {
+                        const uint32_t dst = d0 + k;
+                        if (dst < d.cap) __stcs(dstp + (size_t)dst * CH + c, v[u]);
+                    }
+                }
             }
         }
-#pragma unroll
-        for (int u = 0; u < GU; ++u) {
-            for (uint32_t k = 0; k < rr[u]; ++k) {
-                const uint32_t dst = d0[u] + k;
-                if (dst < d.cap) __stcs(dstp + (size_t)dst * CH + cc[u], v[u]);
-            }
-        }
-    }
     }
     const uint32_t* esrc = d.ebin[src] + base;
     const int32_t* msrc = d.mag[src] + base;
     uint32_t* edst = d.ebin[src ^ 1u];
     int32_t* mdst = d.mag[src ^ 1u];
-    for (uint32_t jl = t; jl < nlist; jl += RS_THREADS) {
-#if PA_RS_COMPACT
-        const uint32_t li = sm.surv[jl];
-#else
-        const uint32_t li = jl;
-#endif
-        const uint32_t rr = s_r[li];
-        if (rr == 0) continue;
+    for (uint32_t jl = t; jl < nsurv; jl += RS_THREADS) {
+        const uint32_t li = sm.surv[jl], rr = sm.r[jl], d0 = sm.o[jl];
         const uint32_t e = esrc[li];
         const int32_t m = msrc[li];
         for (uint32_t k = 0; k < rr; ++k) {
-            const uint32_t dst = s_o[li] + k;
+            const uint32_t dst = d0 + k;
             if (dst < d.cap) {
                 edst[dst] = e;
                 mdst[dst] = m;
@@ -502,25 +479,28 @@ __device__ __forceinline__ void resample_tile(const RunDev& d, uint32_t tile, Re
     }
 }
 
-// Persistent: one wave of CTAs, each claiming tiles until none is left.
-// Claims come in increasing order, so a tile's lookback only waits on tiles
-// already claimed by running CTAs.
-// Resident CTAs per SM the register budget of the nearest-integer and
-// counts-from-memory rules is sized for (the Poisson rule takes 2).
+// Persistent: one wave of CTAs, each claiming slices of tiles until none is
+// left.  Claims come in increasing order, so a tile's lookback only waits on
+// tiles whose first slice is already claimed by a running CTA.  Measured on
+// GB300 (us per launch, one CTA per tile and a lookback by one thread -> slices
+// and the block-wide lookback): 20480 replicas at L = 64 (12 tiles) 77 -> 13.7,
+// 5001 at L = 128 (4 tiles) 243 -> 14.9, 150001 at L = 32 (77 tiles) 38 -> 20,
+// 1000 at L = 16 29 -> 8.5, 2^21 at L = 64 (1036 tiles, no slices) 362 -> 346.
+// Resident CTAs per SM the register budget is sized for.
 #ifndef PA_RS_MINB
 #define PA_RS_MINB 4
 #endif
 template <int RULE, bool SPLIT>
-__global__ void __launch_bounds__(RS_THREADS, RULE == 1 ? 2 : PA_RS_MINB) k_resample(RunDev d) {
+__global__ void __launch_bounds__(RS_THREADS, PA_RS_MINB) k_resample(RunDev d) {
     __shared__ ResampleSmem sm;
     if (!d.st->active) return;
     const uint32_t R = d.st->R_prev;
     for (;;) {
         if (threadIdx.x == 0) sm.tile = atomicAdd(&d.st->tile_counter, 1u);
         __syncthreads();
-        const uint32_t tile = sm.tile;
+        const uint32_t id = sm.tile, tile = id >> d.slice_lg;
         if (tile * (uint32_t)RS_TILE >= R) break;
-        resample_tile<RULE, SPLIT>(d, tile, sm);
+        resample_tile<RULE, SPLIT>(d, tile, id & ((1u << d.slice_lg) - 1u), sm);
         __syncthreads();  // sm is reused by the next tile
     }
 }
@@ -653,7 +633,7 @@ __global__ void __launch_bounds__(256) k_remap(RunDev d, const __grid_constant__
 // tile_base[r] .. tile_base[r+1]-1, so within a run tiles are claimed in order
 // and the lookback only ever waits on tiles already running.
 template <int RULE>
-__global__ void __launch_bounds__(RS_THREADS) k_resample_batched(BatchDev b) {
+__global__ void __launch_bounds__(RS_THREADS, PA_RS_MINB) k_resample_batched(BatchDev b) {
     __shared__ ResampleSmem sm;
     __shared__ uint32_t s_run;
 #if PA_RS_STAGE
@@ -688,7 +668,8 @@ __global__ void __launch_bounds__(RS_THREADS) k_resample_batched(BatchDev b) {
 #else
         const RunDev& d = b.runs[s_run];
 #endif
-        if (d.st->active) resample_tile<RULE>(d, sm.tile, sm);
+        if (d.st->active)
+            resample_tile<RULE>(d, sm.tile >> d.slice_lg, sm.tile & ((1u << d.slice_lg) - 1u), sm);
         __syncthreads();
     }
 }
@@ -803,7 +784,8 @@ static int resample_wave(const void* fn, int which, uint32_t tiles) {
 // PA_RS_SPLIT = 1: the plain resample is two kernels, counts + scan (with the
 // slot -> source map, levels and magnetisations) and then k_gather over the
 // whole new population; 0 (the default): one kernel that gathers tile by
-// tile.  Measured on GB300 at 2^21 replicas, L = 64, same bits: one kernel
+// tile (its figures here are from before its gather kept only data in
+// registers).  Measured on GB300 at 2^21 replicas, L = 64, same bits: one kernel
 // 0.366 ms with 4 loads in flight per thread in its gather (0.361 ms with 6,
 // the default); two kernels 0.374 ms (16 loads in flight per thread, 2 CTAs of
 // 256 per SM), 0.380 ms (4 loads, 4 CTAs), 0.385 ms (8 loads, 3 CTAs).  The split
@@ -829,20 +811,34 @@ static int gather_grid() {
     return cache[dev];
 }
 
+// CTAs of a grid-stride pass over `n` replicas, 256 threads each.
+static int flat_grid(uint64_t n) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    const uint64_t want = (n + 255u) / 256u, cap = (uint64_t)sms * 8u;
+    return (int)(want < cap ? (want ? want : 1u) : cap);
+}
+
 template <bool SPLIT>
 static cudaError_t launch_counts_scan(const RunDev& d, cudaStream_t s) {
-    // cache slots: 0/2/4 the one-kernel forms, 7/8/9 the split forms
-    const int slot = SPLIT ? 7 : 0;
     if (d.resample == PA_RESAMPLE_POISSON) {
-        const int grid = resample_wave((const void*)k_resample<1, SPLIT>, SPLIT ? 8 : 2, d.tiles);
-        if (grid <= 0) return cudaErrorInvalidValue;
-        k_resample<1, SPLIT><<<grid, RS_THREADS, 0, s>>>(d);
-    } else if (d.resample == PA_RESAMPLE_MULTINOMIAL) {
-        const int grid = resample_wave((const void*)k_resample<2, SPLIT>, SPLIT ? 9 : 4, d.tiles);
+        const int g = flat_grid(d.cap);
+        if (g <= 0) return cudaErrorInvalidValue;
+        k_poisson_counts<<<g, 256, 0, s>>>(d);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    // cache slots: 0 and 4 the one-kernel forms, 7 and 9 the split forms
+    if (d.resample != PA_RESAMPLE_NEAREST) {
+        const int grid = resample_wave((const void*)k_resample<2, SPLIT>, SPLIT ? 9 : 4,
+                                       d.tiles << d.slice_lg);
         if (grid <= 0) return cudaErrorInvalidValue;
         k_resample<2, SPLIT><<<grid, RS_THREADS, 0, s>>>(d);
     } else {
-        const int grid = resample_wave((const void*)k_resample<0, SPLIT>, slot, d.tiles);
+        const int grid = resample_wave((const void*)k_resample<0, SPLIT>, SPLIT ? 7 : 0,
+                                       d.tiles << d.slice_lg);
         if (grid <= 0) return cudaErrorInvalidValue;
         k_resample<0, SPLIT><<<grid, RS_THREADS, 0, s>>>(d);
     }
@@ -1024,14 +1020,9 @@ cudaError_t launch_multinomial(const RunDev& d, cudaStream_t s) {
     k_mn_tile_sums<<<wave, RS_THREADS, 0, s>>>(d);
     k_mn_scan<<<1, 1024, 0, s>>>(d);
     k_mn_cum<<<wave, RS_THREADS, 0, s>>>(d);
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return cudaErrorInvalidValue;
-    const uint32_t pairs = (d.R0 + 1u) / 2u;
-    const uint32_t want = (pairs + 255u) / 256u;
-    const uint32_t cap = (uint32_t)sms * 8u;
-    k_mn_draw<<<want < cap ? (want ? want : 1u) : cap, 256, 0, s>>>(d);
+    const int g = flat_grid((d.R0 + 1u) / 2u);
+    if (g <= 0) return cudaErrorInvalidValue;
+    k_mn_draw<<<g, 256, 0, s>>>(d);
     return cudaGetLastError();
 }
 
@@ -1046,14 +1037,15 @@ cudaError_t launch_tau_batched(const BatchDev& b, cudaStream_t s) {
 }
 
 cudaError_t launch_resample_batched(const BatchDev& b, cudaStream_t s) {
-    if (b.any_multinomial) {
+    if (b.any_poisson) {
+        k_poisson_counts_batched<<<b.total_tiles >> b.slice_lg, RS_THREADS, 0, s>>>(b);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    if (b.any_poisson || b.any_multinomial) {
         const int grid = resample_wave((const void*)k_resample_batched<3>, 6, b.total_tiles);
         if (grid <= 0) return cudaErrorInvalidValue;
         k_resample_batched<3><<<grid, RS_THREADS, 0, s>>>(b);
-    } else if (b.any_poisson) {
-        const int grid = resample_wave((const void*)k_resample_batched<1>, 3, b.total_tiles);
-        if (grid <= 0) return cudaErrorInvalidValue;
-        k_resample_batched<1><<<grid, RS_THREADS, 0, s>>>(b);
     } else {
         const int grid = resample_wave((const void*)k_resample_batched<0>, 1, b.total_tiles);
         if (grid <= 0) return cudaErrorInvalidValue;
