@@ -460,22 +460,21 @@ void pa_batch_free(pa_batch* batch);
  * `step` under `seed` and `instance_id`, so the output equals the counts and
  * offsets pa_resample computes for the same population.
  *
- * It allocates nothing: the scratch of its single-pass scan lives in a static
- * device array of about 33 KB that every GPU loading this library holds until
+ * It allocates nothing: the scratch of its scan lives in a static
+ * device array of 32 KB that every GPU loading this library holds until
  * the process exits.  R may be at most PA_NOALLOC_MAX_REPLICAS; larger R (or a
  * negative one, NULL pointers, bins < 1, a negative step or an instance id
  * >= 2^28) returns PA_ERR_INVALID_ARG before anything is enqueued.
  * The first call in each CUDA context (a device's primary context, or a
  * context the caller created and made current) looks up the array's address
  * in that context and caches it under the context's id; make that first call
- * before any stream capture.  Every call reuses the same array and clears what
- * it reads before writing it (the tile counter, the status bits and the
- * lookback descriptors of its tiles), so nothing an earlier call left behind
- * can leak into its result; but two calls whose kernels overlap on the GPU --
- * on different streams, or from different threads -- race and give wrong
- * results: serialise them.
+ * before any stream capture.  Every call reuses the same array and writes the
+ * entries of its tiles before it reads them, so nothing an earlier call left
+ * behind can leak into its result; but two calls whose kernels overlap on the
+ * GPU -- on different streams, or from different threads -- race and give
+ * wrong results: serialise them.
  * *d_total reads 0xFFFFFFFF if a level was >= bins (that replica counts 0
- * copies) or if a bounded wait inside the scan gave up. */
+ * copies). */
 #define PA_NOALLOC_MAX_REPLICAS 8388608
 int pa_copy_counts_scan_noalloc(const uint32_t* d_ebin, int64_t R, const uint32_t* d_tab_n,
                                 const uint32_t* d_tab_F, int64_t bins, uint64_t seed,
