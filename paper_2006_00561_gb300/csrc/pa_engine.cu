@@ -1421,6 +1421,9 @@ int batch_init(pa_run* const* runs, int32_t nruns, const int32_t* steps_left, vo
     b->bd.tile_base = d_tile_base;
     b->bd.total_tiles = tile_base.back();
     b->bd.slice_lg = slice_lg;
+    b->bd.max_bins = 1;
+    for (const auto& h : h_runs)
+        if (h.bins > b->bd.max_bins) b->bd.max_bins = h.bins;
     b->bd.any_poisson = 0;
     b->bd.any_multinomial = 0;
     for (const auto& h : h_runs) {

@@ -5,6 +5,7 @@
 // be enqueued or replayed from a CUDA graph without any host round trip.
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -51,7 +52,9 @@ struct DevState {
 static_assert(sizeof(DevState) <= 256, "DevState must fit its slot");
 
 // Per-step record, same layout as pa_obs.
-static_assert(sizeof(pa_obs) == 104, "pa_obs layout");
+static_assert(sizeof(pa_obs) == 104 && offsetof(pa_obs, sumM2) - offsetof(pa_obs, sumE) == 24 &&
+                  offsetof(pa_obs, chi) - offsetof(pa_obs, e) == 24,
+              "pa_obs layout (the sums and the averages are four in a row)");
 
 // Everything a kernel needs, passed by value.
 struct RunDev {
@@ -109,6 +112,7 @@ struct RunDev {
 struct BatchDev {
     const RunDev* runs;          // [nruns]
     uint32_t nruns;
+    int64_t max_bins;            // energy levels of the run with the most
     const uint32_t* tile_base;   // [nruns + 1] prefix sums of each run's slices of tiles
     uint32_t total_tiles;        // slices of all tiles
     uint32_t slice_lg;           // log2 of the slices of a tile (every run's RunDev::slice_lg)

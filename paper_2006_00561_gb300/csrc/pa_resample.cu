@@ -1,7 +1,7 @@
 // pa_resample.cu -- reweighting and resampling of the population (Sec. 2,
 // Eq. 3 and Eq. 4) and the per-step observables (Sec. 2, Eq. 5).
 //
-//  k_tau       up to 16 CTAs: the energy histogram H of the population at beta_{i-1}
+//  k_tau       up to 33 CTAs: the energy histogram H of the population at beta_{i-1}
 //              gives kref (lowest occupied level when cooling, highest when
 //              heating), S = sum_k H_k D[|k - kref|] with D[j] =
 //              exp(-|beta_i - beta_{i-1}| 4 j), Q = S exp(-dbeta E(kref)) / R
@@ -40,84 +40,148 @@ __device__ __forceinline__ void stage_run(const RunDev* src, RunDev& dst) {
     for (uint32_t w = threadIdx.x; w < sizeof(RunDev) / 4; w += blockDim.x) to[w] = from[w];
 }
 
-// Reweight of one run by nblk 256-thread CTAs (plain: k_tau, batched: one
-// CTA per run of k_tau_batched).  Every CTA finds kref and S itself (the same
-// fixed order, so the same bits) and writes the tau entries of its share of
-// the levels; the last CTA to finish, when every CTA has read the step index
-// and R, advances the run's scalars.
-__device__ __forceinline__ void tau_run(const RunDev& d, uint32_t blk, uint32_t nblk) {
+// Calls f(k, H_k) for the occupied levels of the thread's share of the
+// histogram (four consecutive levels of every 4 * 256).
+template <typename F>
+__device__ __forceinline__ void each_level(const uint32_t* hist, uint32_t bins, F&& f) {
+    const uint4* h4 = reinterpret_cast<const uint4*>(hist);  // 16-byte aligned
+    const uint32_t quads = bins >> 2;
+#pragma unroll 4
+    for (uint32_t q = threadIdx.x; q < quads; q += 256) {
+        const uint4 h = h4[q];
+        if (h.x) f(4 * q, h.x);
+        if (h.y) f(4 * q + 1, h.y);
+        if (h.z) f(4 * q + 2, h.z);
+        if (h.w) f(4 * q + 3, h.w);
+    }
+    const uint32_t k = 4 * quads + threadIdx.x;
+    if (k < bins) {
+        const uint32_t h = hist[k];
+        if (h) f(k, h);
+    }
+}
+
+// Reweight of one run by nblk 256-thread CTAs.  Every CTA finds kref and S
+// itself (the same fixed order, so the same bits) and writes the tau entries
+// of its share of the levels; the last CTA to finish, when every CTA has read
+// the step index and R, advances the run's scalars.  Returns whether this CTA
+// is the one that was last to read the histogram.
+//
+// Bound: GB300 retires about two FP64 operations per SM and clock, so the
+// latency is the FP64 work of one CTA.  Hence levels without replicas add
+// nothing (x + 0 * D is x, exactly) and are skipped, levels whose tau is below
+// 2^-33 get (0, 0) without a division, more CTAs share the divisions, and the
+// two logarithms run in a warp of their own beside them.  Before -> after, timed
+// by events: 13.4 -> 12.2 us (257 levels), 25 -> 14.7 (4097), 44 -> 24 (16385); a
+// batch of 28 runs with up to 16385 levels 87 -> 39.
+constexpr uint32_t TAU_LEVELS = 128;  // levels per CTA and pass
+// CTAs of a run at most: 33, 65 and 130 run alike on GB300 (14.7 us at 4097
+// levels, 24 us at 16385, timed by events around the launch).
+#ifndef PA_TAU_CTAS
+#define PA_TAU_CTAS 33
+#endif
+constexpr uint32_t TAU_CTAS = PA_TAU_CTAS;
+__device__ __forceinline__ bool tau_run(const RunDev& d, uint32_t blk, uint32_t nblk) {
     DevState* st = d.st;
-    __shared__ double part[256];
-    __shared__ uint32_t s_kref;
+    __shared__ double s_part[8];
+    __shared__ double s_lnR;
+    __shared__ uint32_t s_min[8], s_max[8];
     __shared__ unsigned long long s_sum;
-    const int t = threadIdx.x;
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const uint32_t i = st->step + 1;
     const uint32_t R = st->R;
     const uint32_t bins = (uint32_t)d.bins;
     if (i > (uint32_t)d.K || R == 0) {
-        if (t == 0) {
+        if (t == 0 && blk == 0) {
             st->active = 0;
             atomicOr(&st->status, i > (uint32_t)d.K ? ST_DONE : ST_EMPTY);
         }
-        return;
+        return blk == 0;
     }
+    const double db = d.dbeta[i];
+    const double* __restrict__ D = d.dtab + (size_t)d.dsel[i] * bins;
     // reference level: lowest occupied when cooling, highest when heating
-    const bool heating = d.dbeta[i] < 0.0;
-    if (t == 0) {
-        s_kref = heating ? 0u : 0xffffffffu;
-        s_sum = 0;
-    }
-    __syncthreads();
-    uint32_t kext = heating ? 0u : 0xffffffffu;
-    bool any = false;
+    const bool heating = db < 0.0;
+    if (t == 0) s_sum = 0;
+    uint32_t kmin = 0xffffffffu, kmax = 0u;
     unsigned long long hs = 0;
-    for (uint32_t k = t; k < bins; k += 256) {
-        const uint32_t h = d.hist[k];
-        if (h) {
-            any = true;
-            kext = heating ? (k > kext ? k : kext) : (k < kext ? k : kext);
-        }
+    each_level(d.hist, bins, [&](uint32_t k, uint32_t h) {
+        kmin = min(kmin, k);
+        kmax = max(kmax, k);
         hs += h;
+    });
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0) {
+        s_min[wid] = kmin;
+        s_max[wid] = kmax;
     }
-    if (heating) {
-        if (any) atomicMax(&s_kref, kext);
-    } else {
-        atomicMin(&s_kref, kext);
-    }
-    atomicAdd(&s_sum, hs);
+    const bool logs = blk == nblk - 1;  // this CTA also takes ln Q and the check of sum H
+    if (logs && t == 160) s_lnR = log((double)R);
     __syncthreads();
-    const uint32_t kref = s_kref;
-    const double* D = d.dtab + (size_t)d.dsel[i] * bins;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        kmin = min(kmin, s_min[w]);
+        kmax = max(kmax, s_max[w]);
+    }
+    const uint32_t kref = heating ? kmax : kmin;
+    if (logs && hs) atomicAdd(&s_sum, hs);
     // S in the fixed order: 256 contiguous chunks summed left to right, then a
     // pairwise tree over the chunk sums; level k weighs D[|k - kref|].
     const uint32_t ch = (bins + 255) / 256;
+    const uint32_t k_lo = max(t * ch, kmin), k_hi = min(min((t + 1) * ch, bins), kmax + 1u);
     double acc = 0.0;
-    for (uint32_t k = t * ch; k < (t + 1) * ch && k < bins; ++k) {
-        const int64_t j = heating ? (int64_t)kref - (int64_t)k : (int64_t)k - (int64_t)kref;
-        if (j >= 0) acc = __dadd_rn(acc, __dmul_rn((double)d.hist[k], D[j]));
-    }
-    part[t] = acc;
-    __syncthreads();
-    for (int w = 256; w > 1; w >>= 1) {
-        double v = 0.0;
-        if (t < w / 2) v = __dadd_rn(part[2 * t], part[2 * t + 1]);
-        __syncthreads();
-        if (t < w / 2) part[t] = v;
-        __syncthreads();
-    }
-    const double S = part[0];
-    const double R0d = (double)d.R0;
-    for (uint32_t k = blk * 256u + t; k < bins; k += nblk * 256u) {
-        uint32_t n = 0, F = 0;
-        const int64_t j = heating ? (int64_t)kref - (int64_t)k : (int64_t)k - (int64_t)kref;
-        if (j >= 0) {
-            const double tau = __ddiv_rn(__dmul_rn(R0d, D[j]), S);
-            const double nk = floor(tau);
-            n = (uint32_t)nk;
-            F = (uint32_t)floor(__dmul_rn(__dsub_rn(tau, nk), 4294967296.0));
+    for (uint32_t k0 = k_lo; k0 < k_hi; k0 += 8) {
+        uint32_t h[8];
+        double w[8];
+#pragma unroll
+        for (uint32_t j = 0; j < 8; ++j) {
+            const uint32_t k = k0 + j;
+            h[j] = 0;
+            if (k < k_hi) {
+                h[j] = d.hist[k];
+                w[j] = D[heating ? kref - k : k - kref];
+            }
         }
-        d.tab_n[k] = n;
-        d.tab_F[k] = F;
+#pragma unroll
+        for (uint32_t j = 0; j < 8; ++j)
+            if (h[j]) acc = __dadd_rn(acc, __dmul_rn((double)h[j], w[j]));
+    }
+    if (__any_sync(0xffffffffu, acc != 0.0)) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) acc = __dadd_rn(acc, __shfl_xor_sync(0xffffffffu, acc, o));
+    }
+    if (lane == 0) s_part[wid] = acc;
+    __syncthreads();
+    const double S = __dadd_rn(
+        __dadd_rn(__dadd_rn(s_part[0], s_part[1]), __dadd_rn(s_part[2], s_part[3])),
+        __dadd_rn(__dadd_rn(s_part[4], s_part[5]), __dadd_rn(s_part[6], s_part[7])));
+    if (wid < 4) {
+        const double R0d = (double)d.R0;
+        const double least = __dmul_rn(S, 5.8207660913467407e-11);  // 2^-34 S: tau < 2^-33
+        for (uint32_t k = blk * TAU_LEVELS + t; k < bins; k += nblk * TAU_LEVELS) {
+            uint32_t n = 0, F = 0;
+            const int64_t j = heating ? (int64_t)kref - (int64_t)k : (int64_t)k - (int64_t)kref;
+            if (j >= 0) {
+                const double w = __dmul_rn(R0d, D[j]);
+                if (!(w < least)) {
+                    const double tau = __ddiv_rn(w, S);
+                    const double nk = floor(tau);
+                    n = (uint32_t)nk;
+                    F = (uint32_t)floor(__dmul_rn(__dsub_rn(tau, nk), 4294967296.0));
+                }
+            }
+            d.tab_n[k] = n;
+            d.tab_F[k] = F;
+        }
+    } else if (logs && t == 128) {
+        if (s_sum != (unsigned long long)R) atomicOr(&st->status, ST_INVARIANT);
+        const long long parity = st->negbonds & 1u;
+        const long long Eref = 2 * (2 * (long long)kref + parity) - (long long)d.dim * d.N;
+        const double lnQ = __dsub_rn(__dsub_rn(log(S), s_lnR), __dmul_rn(db, (double)Eref));
+        st->lnQ = lnQ;
+        st->lnZ = __dadd_rn(st->lnZ, lnQ);
+        st->S = S;
     }
     if (nblk > 1) {
         __shared__ bool s_last;
@@ -127,45 +191,47 @@ __device__ __forceinline__ void tau_run(const RunDev& d, uint32_t blk, uint32_t 
             s_last = atomicAdd(&st->tau_done, 1ull) == (unsigned long long)(nblk - 1);
         }
         __syncthreads();
-        if (!s_last) return;
+        if (!s_last) return false;
     }
     if (t == 0) {
         st->tau_done = 0;
-        if (s_sum != (unsigned long long)R) atomicOr(&st->status, ST_INVARIANT);
-        const long long parity = st->negbonds & 1u;
-        const long long Eref = 2 * (2 * (long long)kref + parity) - (long long)d.dim * d.N;
-        const double lnQ =
-            __dsub_rn(__dsub_rn(log(S), log((double)R)), __dmul_rn(d.dbeta[i], (double)Eref));
-        st->lnQ = lnQ;
-        st->lnZ = __dadd_rn(st->lnZ, lnQ);
-        st->S = S;
         st->kref = kref;
         st->step = i;
         st->R_prev = R;
         st->epoch = st->epoch + 1;
         st->tile_counter = 0;
-        st->src = st->cur;
-        st->cur = st->cur ^ 1u;
+        const uint32_t cur = st->cur;
+        st->src = cur;
+        st->cur = cur ^ 1u;
         st->active = 1;
     }
+    return true;
 }
 
-__global__ void __launch_bounds__(256) k_tau(RunDev d) { tau_run(d, blockIdx.x, gridDim.x); }
+__global__ void __launch_bounds__(256) k_tau(__grid_constant__ const RunDev d) {
+    tau_run(d, blockIdx.x, gridDim.x);
+}
 
-// Batched reweight: CTA r handles run r, then clears that run's histogram and
-// magnetisation sums for the coming sweep (the reweight is their last
-// reader); CTA 0 clears the batch's work counters.
+// CTAs of a run's reweight: one per TAU_LEVELS levels, at most TAU_CTAS.
+__host__ __device__ inline uint32_t tau_ctas(int64_t bins) {
+    const int64_t per = (bins + TAU_LEVELS - 1) / TAU_LEVELS;
+    return per < 1 ? 1u : per < (int64_t)TAU_CTAS ? (uint32_t)per : TAU_CTAS;
+}
+
+// Batched reweight: column r of the grid handles run r, whose last CTA then clears
+// the run's histogram and magnetisation sums for the coming sweep (the
+// reweight is their last reader); the first CTA clears the batch's work
+// counters.
 __global__ void __launch_bounds__(256) k_tau_batched(BatchDev b) {
-    if (blockIdx.x == 0 && threadIdx.x < b.ncounters) b.counters[threadIdx.x] = 0u;
-#if PA_RS_STAGE
+    if (blockIdx.x == 0 && blockIdx.y == 0)
+        for (uint32_t c = threadIdx.x; c < b.ncounters; c += 256) b.counters[c] = 0u;
+    const uint32_t nblk = tau_ctas(b.runs[blockIdx.x].bins);
+    if (blockIdx.y >= nblk) return;
     __shared__ RunDev s_d;
     stage_run(&b.runs[blockIdx.x], s_d);
     __syncthreads();
     const RunDev& d = s_d;
-#else
-    const RunDev& d = b.runs[blockIdx.x];
-#endif
-    tau_run(d, 0, 1);
+    if (!tau_run(d, blockIdx.y, nblk)) return;
     __syncthreads();
     for (uint32_t k = threadIdx.x; k < (uint32_t)d.bins; k += blockDim.x) d.hist[k] = 0u;
     if (threadIdx.x < 2) d.accum[threadIdx.x] = 0ull;
@@ -680,22 +746,26 @@ __device__ __forceinline__ long long warp_sum_ll(long long v) {
     return v;
 }
 
+// The record of the measured step: integer sums over the histogram by the CTA,
+// then the averages, one per lane of a warp (an FP64 division is a chain of
+// some ten dependent FP64 operations: two of them one after the other instead
+// of eight; 10.0 -> 8.3 us at 4097 levels, timed by events).
 __device__ __forceinline__ void obs_run(const RunDev& d, int nsweeps) {
     DevState* st = d.st;
     __shared__ long long s_part[3][8];
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    const uint32_t step = st->step;
+    const uint32_t step = st->step, R = st->R;
     const long long parity = st->negbonds & 1u;
     const long long dimN = (long long)d.dim * d.N;
+    const double beta = d.beta[step];
     long long cnt = 0, sE = 0, sE2 = 0;
-    for (uint32_t k = t; k < (uint32_t)d.bins; k += 256) {
-        const long long h = d.hist[k];
-        if (!h) continue;
+    each_level(d.hist, (uint32_t)d.bins, [&](uint32_t k, uint32_t h) {
         const long long E = 2 * (2 * (long long)k + parity) - dimN;
+        const long long hE = (long long)h * E;
         cnt += h;
-        sE += h * E;
-        sE2 += h * E * E;
-    }
+        sE += hE;
+        sE2 += hE * E;
+    });
     cnt = warp_sum_ll(cnt);
     sE = warp_sum_ll(sE);
     sE2 = warp_sum_ll(sE2);
@@ -705,40 +775,48 @@ __device__ __forceinline__ void obs_run(const RunDev& d, int nsweeps) {
         s_part[2][wid] = sE2;
     }
     __syncthreads();
-    if (t == 0) {
-        for (int w = 1; w < 8; ++w) {
-            cnt += s_part[0][w];
-            sE += s_part[1][w];
-            sE2 += s_part[2][w];
-        }
-        const uint32_t R = st->R;
-        if (cnt != (long long)R) atomicOr(&st->status, ST_INVARIANT);
-        pa_obs o;
-        o.step = step;
-        o.R = R;
-        o.sumE = sE;
-        o.sumE2 = sE2;
-        o.sumAbsM = (long long)d.accum[0];
-        o.sumM2 = (long long)d.accum[1];
-        o.beta = d.beta[step];
-        o.lnQ = st->lnQ;
-        o.lnZ = st->lnZ;
-        const double Rd = (double)R, Nd = (double)d.N;
-        const double mE = __ddiv_rn((double)o.sumE, Rd);
-        const double mE2 = __ddiv_rn((double)o.sumE2, Rd);
-        const double mA = __ddiv_rn((double)o.sumAbsM, Rd);
-        const double mM2 = __ddiv_rn((double)o.sumM2, Rd);
-        o.e = __ddiv_rn(mE, Nd);
-        o.cv = __ddiv_rn(__dmul_rn(__dmul_rn(o.beta, o.beta), __dsub_rn(mE2, __dmul_rn(mE, mE))), Nd);
-        o.m_abs = __ddiv_rn(mA, Nd);
-        o.chi = __ddiv_rn(__dmul_rn(o.beta, __dsub_rn(mM2, __dmul_rn(mA, mA))), Nd);
-        d.obs[step] = o;
+    if (wid != 0) return;
+    long long p0 = 0, p1 = 0, p2 = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        p0 += s_part[0][w];
+        p1 += s_part[1][w];
+        p2 += s_part[2][w];
+    }
+    // lanes 0..3: sum E, sum E^2, sum |M|, sum M^2 and their averages
+    const long long sum = lane == 0   ? p1
+                          : lane == 1 ? p2
+                          : lane < 4  ? (long long)d.accum[lane - 2]
+                                      : 0ll;
+    const double Nd = (double)d.N;
+    const double mean = __ddiv_rn((double)sum, (double)R);
+    const double mE = __shfl_sync(0xffffffffu, mean, 0), mE2 = __shfl_sync(0xffffffffu, mean, 1);
+    const double mA = __shfl_sync(0xffffffffu, mean, 2), mM2 = __shfl_sync(0xffffffffu, mean, 3);
+    // lanes 0..3: e, cv, m_abs, chi
+    const double num =
+        lane == 0   ? mE
+        : lane == 1 ? __dmul_rn(__dmul_rn(beta, beta), __dsub_rn(mE2, __dmul_rn(mE, mE)))
+        : lane == 2 ? mA
+                    : __dmul_rn(beta, __dsub_rn(mM2, __dmul_rn(mA, mA)));
+    const double avg = __ddiv_rn(num, Nd);
+    pa_obs* o = d.obs + step;
+    if (lane < 4) {
+        (&o->sumE)[lane] = sum;
+        (&o->e)[lane] = avg;
+    }
+    if (lane == 0) {
+        if (p0 != (long long)R) atomicOr(&st->status, ST_INVARIANT);
+        o->step = step;
+        o->R = R;
+        o->beta = beta;
+        o->lnQ = st->lnQ;
+        o->lnZ = st->lnZ;
         st->sweep_base = st->sweep_base + (uint32_t)nsweeps;
         st->sweeps_done = st->sweeps_done + (unsigned long long)nsweeps;
     }
 }
 
-__global__ void __launch_bounds__(256) k_obs(RunDev d, int nsweeps) { obs_run(d, nsweeps); }
+__global__ void __launch_bounds__(256) k_obs(__grid_constant__ const RunDev d, int nsweeps) { obs_run(d, nsweeps); }
 
 __global__ void __launch_bounds__(256) k_obs_batched(BatchDev b) {
 #if PA_RS_STAGE
@@ -754,12 +832,8 @@ __global__ void __launch_bounds__(256) k_obs_batched(BatchDev b) {
 
 }  // namespace
 
-// CTAs of the plain reweight: one per 256 levels, at most 16 (the tau
-// divisions are FP64; each CTA also repeats the sum S, 16 FP64 terms a thread).
 cudaError_t launch_tau(const RunDev& d, cudaStream_t s) {
-    const int64_t per = ((int64_t)d.bins + 255) / 256;
-    const int grid = (int)(per < 16 ? per : 16);
-    k_tau<<<grid < 1 ? 1 : grid, 256, 0, s>>>(d);
+    k_tau<<<tau_ctas(d.bins), 256, 0, s>>>(d);
     return cudaGetLastError();
 }
 
@@ -1032,7 +1106,7 @@ cudaError_t launch_obs(const RunDev& d, int nsweeps, cudaStream_t s) {
 }
 
 cudaError_t launch_tau_batched(const BatchDev& b, cudaStream_t s) {
-    k_tau_batched<<<b.nruns, 256, 0, s>>>(b);
+    k_tau_batched<<<dim3(b.nruns, tau_ctas(b.max_bins)), 256, 0, s>>>(b);
     return cudaGetLastError();
 }
 
