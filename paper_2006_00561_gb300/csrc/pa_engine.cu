@@ -1359,6 +1359,7 @@ int batch_init(pa_run* const* runs, int32_t nruns, const int32_t* steps_left, vo
         d.slice_lg = slice_lg;
         tile_base.push_back(tile_base.back() + (d.tiles << slice_lg));
     }
+    const int sliced_warps = pa::batched_default_warps(h_runs.data(), nruns);
     // classes: one sweep kernel instantiation per (layout, dim, L, model)
     for (int32_t i = 0; i < nruns; ++i) {
         const pa::RunDev& d = h_runs[i];
@@ -1374,7 +1375,7 @@ int batch_init(pa_run* const* runs, int32_t nruns, const int32_t* steps_left, vo
             k.L = d.L;
             k.model = d.model;
             k.proto = d;
-            k.warps = pa::l64_batched_applies(d) ? pa::l64_block_warps(d) : 4;
+            k.warps = pa::l64_batched_applies(d) ? pa::l64_block_warps(d) : sliced_warps;
             k.stream = nullptr;
             k.done = nullptr;
             b->cls.push_back(k);

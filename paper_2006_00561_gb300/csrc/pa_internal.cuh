@@ -286,13 +286,15 @@ cudaError_t launch_philox_rate(uint64_t seed, uint32_t halfsweeps, uint32_t* out
 cudaError_t launch_tau_batched(const BatchDev& b, cudaStream_t s);
 cudaError_t launch_resample_batched(const BatchDev& b, cudaStream_t s);
 cudaError_t launch_obs_batched(const BatchDev& b, cudaStream_t s);
-// sweep of one class; `warps` selects the block shape (an autotuned knob:
-// 2, 4 or 8 warps per block for the shared-memory kernels; the L = 64
-// register kernel has one shape), grid 0 = one wave of resident blocks
+// sweep of one class; `warps` selects the block shape (an autotuned knob: 2, 4
+// or 8 for the replica-sliced kernel; the register kernels have one shape),
+// grid: one wave of resident blocks
 cudaError_t launch_sweep_batched(const BatchSweepArgs& a, const RunDev& proto, int warps, int grid,
                                  cudaStream_t s);
 int batched_sweep_grid(const RunDev& proto, int warps);
 bool batched_warps_valid(const RunDev& proto, int warps);
+// the shape of the replica-sliced classes of a batch of these runs
+int batched_default_warps(const RunDev* runs, int n);
 bool l64_batched_applies(const RunDev& proto);
 cudaError_t launch_sweep_l64_batched(const BatchSweepArgs& a, const RunDev& proto, int grid,
                                      cudaStream_t s);
