@@ -725,16 +725,13 @@ __global__ void __launch_bounds__(Team<DIM, L, RSP>::TT) k_sweep_team_batched(Ba
 // bond (s, d): top bit of word s & 3 of (s >> 2, d, 0, COUPLING | instance)
 // under the coupling key; set means J = -1.
 // --------------------------------------------------------------------------
-__global__ void k_init_packed(RunDev d, int nrows, int NW) {
+// Packed rows of any even length: one thread per word and replica.
+__global__ void k_init_packed(RunDev d, int NW) {
     const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t total = (uint64_t)d.R0 * d.nwords;
     if (gid >= total) return;
     const uint32_t slot = (uint32_t)(gid / d.nwords);
     const uint32_t w = (uint32_t)(gid % d.nwords);
-    if (d.init == PA_INIT_GROUND) {  // all spins +1
-        reinterpret_cast<uint32_t*>(d.spins[0] + (size_t)slot * d.stride)[w] = 0u;
-        return;
-    }
     const int r = (int)(w / NW), k = (int)(w % NW);
     const uint32_t ctr3 = (TAG_INIT << 28) | d.instance;
     const uint32_t k0 = (uint32_t)d.seed, k1 = (uint32_t)(d.seed >> 32);
@@ -752,7 +749,63 @@ __global__ void k_init_packed(RunDev d, int nrows, int NW) {
         bits |= (pick(u, (uint32_t)(s & 3)) >> 31) << b;
     }
     reinterpret_cast<uint32_t*>(d.spins[0] + (size_t)slot * d.stride)[w] = bits;
-    (void)nrows;
+}
+
+// The same for rows that are whole Philox blocks (L a multiple of 4): a thread
+// keeps one word of the replica, NB blocks, and walks over the replicas.  The
+// block index enters word 0 and the slot word 2, so the products of rounds 1
+// and 2 each belong to a block (held in registers over all replicas) or to a
+// replica (two per word): a block costs 16 + 2 / NB multiplies instead of 20.
+// Bound by them: the creation of a run of 2^21 replicas of L = 64, with its first
+// measurement, takes 5.6 ms on GB300; with one thread per word and replica (a
+// 64-bit division, and every product of every block) it took 13.6 ms.
+template <int NB>
+__global__ void __launch_bounds__(256) k_init_words(__grid_constant__ const RunDev d) {
+    const uint32_t per = 256u / d.nwords;  // replicas of a block's pass (0: part of one)
+    uint32_t w, first, step;
+    if (per) {
+        w = threadIdx.x % d.nwords;
+        const uint32_t sub = threadIdx.x / d.nwords;
+        if (sub >= per) return;
+        first = blockIdx.x * per + sub;
+        step = gridDim.x * per;
+    } else {
+        w = blockIdx.y * 256u + threadIdx.x;
+        if (w >= d.nwords) return;
+        first = blockIdx.x;
+        step = gridDim.x;
+    }
+    const uint32_t ctr3 = (TAG_INIT << 28) | d.instance;
+    uint32_t h2[NB], l2[NB], l1[NB];  // block halves: round 2 (high, low), round 1 (low)
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+        uint32_t h1;
+        mul_hilo(PM0, w * NB + (uint32_t)j, h1, l1[j]);
+        mul_hilo(PM1, h1 ^ ctr3 ^ d.rk1[0], h2[j], l2[j]);
+    }
+    for (uint32_t slot = first; slot < d.R0; slot += step) {
+        uint32_t hs, ls, hr, lr;  // replica halves
+        mul_hilo(PM1, slot, hs, ls);            // round 1
+        mul_hilo(PM0, hs ^ d.rk0[0], hr, lr);   // round 2
+        uint32_t bits = 0;
+#pragma unroll
+        for (int j = 0; j < NB; ++j) {
+            uint32_t c0 = h2[j] ^ ls ^ d.rk0[1], c1 = l2[j], c2 = hr ^ l1[j] ^ d.rk1[1], c3 = lr;
+#pragma unroll
+            for (int r = 2; r < 10; ++r) {
+                uint32_t hiA, loA, hiB, loB;
+                mul_hilo(PM0, c0, hiA, loA);
+                mul_hilo(PM1, c2, hiB, loB);
+                c0 = hiB ^ c1 ^ d.rk0[r];
+                c1 = loB;
+                c2 = hiA ^ c3 ^ d.rk1[r];
+                c3 = loA;
+            }
+            const uint32_t nib = (c0 >> 31) | (c1 >> 31) << 1 | (c2 >> 31) << 2 | (c3 >> 31) << 3;
+            bits |= nib << (4 * j);
+        }
+        reinterpret_cast<uint32_t*>(d.spins[0] + (size_t)slot * d.stride)[w] = bits;
+    }
 }
 
 __global__ void k_init_i8(RunDev d) {
@@ -961,10 +1014,24 @@ cudaError_t launch_init(const RunDev& d, cudaStream_t s) {
                                                         : (uint64_t)d.N * d.dim;
         k_init_couplings<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(d, NW);
     }
-    if (d.layout == PA_LAYOUT_PACKED) {
+    if (d.layout == PA_LAYOUT_PACKED && d.init == PA_INIT_GROUND) {  // all spins +1
+        const cudaError_t e = cudaMemsetAsync(d.spins[0], 0, (size_t)d.R0 * d.stride, s);
+        if (e != cudaSuccess) return e;
+    } else if (d.layout == PA_LAYOUT_PACKED && d.L % 4 == 0) {
+        // about eight blocks of 256 threads per SM
+        const uint32_t per = 256u / d.nwords, parts = per ? 1u : (d.nwords + 255u) / 256u;
+        const uint32_t passes = per ? (d.R0 + per - 1) / per : d.R0, most = 1216u / parts;
+        const dim3 grid(passes < most ? passes : most, parts);
+        switch (d.L < 32 ? d.L / 4 : 8) {
+            case 1: k_init_words<1><<<grid, 256, 0, s>>>(d); break;
+            case 2: k_init_words<2><<<grid, 256, 0, s>>>(d); break;
+            case 3: k_init_words<3><<<grid, 256, 0, s>>>(d); break;
+            case 4: k_init_words<4><<<grid, 256, 0, s>>>(d); break;
+            default: k_init_words<8><<<grid, 256, 0, s>>>(d); break;
+        }
+    } else if (d.layout == PA_LAYOUT_PACKED) {
         const uint64_t n = (uint64_t)d.R0 * d.nwords;
-        const int nrows = d.dim == 2 ? d.L : d.L * d.L;
-        k_init_packed<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(d, nrows, NW);
+        k_init_packed<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(d, NW);
     } else {
         const uint64_t n = (uint64_t)d.R0 * ((d.N + 3) / 4);
         k_init_i8<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(d);
