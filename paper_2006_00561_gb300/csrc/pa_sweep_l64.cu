@@ -28,12 +28,13 @@
 // device memory.  The measurement epilogue is the one of the generic kernel.
 #include "pa_internal.cuh"
 
+#include <cmath>
+
 namespace pa {
 namespace {
 
-// Tuning knobs (compile time): warps per block and the resident blocks per SM
-// the register budget is sized for; the forms of the threshold tests are the
-// PA_L64_CHAIN and PA_L64_SEL_BLOCKS knobs further down.
+// Tuning knobs (compile time): warps per block; the forms of the threshold
+// tests are the PA_L64_CHAIN and PA_L64_SEL_BLOCKS knobs further down.
 #ifndef PA_L64_MIN_BLOCKS
 #define PA_L64_MIN_BLOCKS 1
 #endif
@@ -44,16 +45,20 @@ namespace {
 #define PA_L64_MUL_MODE 1
 #endif
 
-// Warps per block (one block per SM).  With both groups of a row unrolled,
-// measured on GB300 (attempts/ns, same bits): 16 warps (125 registers) 1671,
-// 12 warps (152) 1686, 8 warps (212) 1653 (ferromagnet, 2^21 replicas); +-J
-// 2^20: 1626, 1636, 1611; batched, 8 +-J runs of 2^17: 1597, 1632, 1604.
-// With the Philox tables (fewer registers) 16 warps ran at 1755 against 1749
-// (ferromagnet) and 1704 against 1712 (+-J): 12 stays.
+// Warps per block of the batched kernel (one block per SM).  With both groups
+// of a row unrolled, measured on GB300 (attempts/ns, same bits), 8 +-J runs of
+// 2^17: 16 warps (125 registers) 1597, 12 warps (152) 1632, 8 warps (212) 1604.
 #ifndef PA_L64_WARPS
 #define PA_L64_WARPS 12
 #endif
 constexpr int WARPS64 = PA_L64_WARPS;
+// Warps per block of the plain kernels.  Consecutive replicas go to different
+// SMs, so a last round of few replicas runs one or two warps on every SM rather
+// than all warps of a few.  us per launch on GB300 (theta = 10), 12 warps with a
+// block's replicas together -> apart at 8, 12, 16 warps: 256 replicas 50 -> 26, 25,
+// 25; 20480 521 -> 502, 494, 489 (theta = 1: 61 -> 64, 61, 58); 2^20 24596 -> 25201, 24469,
+// 24371; +-J 2^20 25121 -> 25648, 24993, 25092.
+constexpr int WARPS64_FERRO = 16, WARPS64_PMJ = 12;
 
 __device__ __forceinline__ uint64_t shfl64(uint64_t v, int src) {
     const uint32_t lo = __shfl_sync(0xffffffffu, (uint32_t)v, src);
@@ -530,8 +535,8 @@ __device__ __forceinline__ void cta_tables(uint2* tab, uint32_t ctag, uint32_t g
     __syncthreads();
 }
 
-template <bool PMJ, bool T3>
-__global__ void __launch_bounds__(WARPS64 * 32, PA_L64_MIN_BLOCKS)
+template <bool PMJ, bool T3, int W>
+__global__ void __launch_bounds__(W * 32, 1)
     k_sweep_l64(__grid_constant__ const RunDev d, int nsweeps) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     DevState* st = d.st;
@@ -550,9 +555,9 @@ __global__ void __launch_bounds__(WARPS64 * 32, PA_L64_MIN_BLOCKS)
     if constexpr (PMJ) l64_couplings(d, lane, ja, jb);
     const uint32_t parity = st->negbonds & 1u;
     L64Tally tally;
-    const uint32_t nwarps = gridDim.x * WARPS64;
+    const uint32_t nwarps = gridDim.x * W;
     const uint32_t end = min(R, d.slot_hi);
-    for (uint32_t slot = d.slot_lo + blockIdx.x * WARPS64 + wib; slot < end; slot += nwarps) {
+    for (uint32_t slot = d.slot_lo + wib * gridDim.x + blockIdx.x; slot < end; slot += nwarps) {
         int M = 0;
         const uint32_t U =
             l64_replica<PMJ, T3>(K, spins, slot, nsweeps, g0, ctag, t4, t8, full, lane, M, ja, jb);
@@ -639,10 +644,11 @@ __global__ void __launch_bounds__(WARPS64 * 32, PA_L64_MIN_BLOCKS) k_sweep_l64_b
 // block) 1490 against 1508 attempts/ns, and one per CTA (16 KB) 1504-1507
 // (ferromagnet) and 1476-1479 against 1495-1497 (+-J).
 // --------------------------------------------------------------------------
-// Block warps: with two groups unrolled, the ferromagnet runs at 1508 to 1517
-// attempts/ns with 8 warps (183 registers) against 1484 with 12 (166
-// registers) on GB300, 2^19 replicas; the +-J kernel holds eight rows of
-// couplings more and keeps 8 warps (12 spill).
+// Block warps of the batched kernel and of the plain +-J one: with two groups
+// unrolled, the ferromagnet runs at 1508 to 1517 attempts/ns with 8 warps (183
+// registers) against 1484 with 12 (166 registers) on GB300, 2^19 replicas; the
+// +-J kernel holds eight rows of couplings more and keeps 8 warps (12 spill).  The
+// plain ferromagnet chooses by the population (warps128_for).
 #ifndef PA_L128_WARPS
 #define PA_L128_WARPS 8
 #endif
@@ -825,8 +831,8 @@ __device__ __forceinline__ uint32_t l128_replica(const Keys& K, uint4* spins, ui
     return U;
 }
 
-template <bool PMJ>
-__global__ void __launch_bounds__(warps128<PMJ>() * 32, 1)
+template <bool PMJ, int W>
+__global__ void __launch_bounds__(W * 32, 1)
     k_sweep_l128(__grid_constant__ const RunDev d, int nsweeps) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     DevState* st = d.st;
@@ -843,10 +849,9 @@ __global__ void __launch_bounds__(warps128<PMJ>() * 32, 1)
     if constexpr (PMJ) l128_couplings(d, lane, j);
     const uint32_t parity = st->negbonds & 1u;
     L64Tally tally;
-    constexpr int W = warps128<PMJ>();
     const uint32_t nwarps = gridDim.x * W;
     const uint32_t end = min(R, d.slot_hi);
-    for (uint32_t slot = d.slot_lo + blockIdx.x * W + wib; slot < end; slot += nwarps) {
+    for (uint32_t slot = d.slot_lo + wib * gridDim.x + blockIdx.x; slot < end; slot += nwarps) {
         int M = 0;
         const uint32_t U =
             l128_replica<PMJ>(K, spins, slot, nsweeps, g0, ctag, t4, t8, full, lane, M, j);
@@ -1001,6 +1006,19 @@ static size_t l64_plain_smem(bool t3, int nsweeps) {
 constexpr size_t L64_BATCHED_SMEM = (size_t)WARPS64 * 16 * 32 * sizeof(uint2);
 constexpr size_t PHILOX_RATE_SMEM = (size_t)(1 + PHILOX_RATE_WIN) * TAB_ROW;
 
+// The plain kernels by model, table form and (L = 128 ferromagnet) warps per block.
+static const void* plain64(bool pmj, bool t3) {
+    if (pmj)
+        return t3 ? (const void*)k_sweep_l64<true, true, WARPS64_PMJ>
+                  : (const void*)k_sweep_l64<true, false, WARPS64_PMJ>;
+    return t3 ? (const void*)k_sweep_l64<false, true, WARPS64_FERRO>
+              : (const void*)k_sweep_l64<false, false, WARPS64_FERRO>;
+}
+static const void* plain128(bool pmj, int w) {
+    if (pmj) return (const void*)k_sweep_l128<true, warps128<true>()>;
+    return w == 12 ? (const void*)k_sweep_l128<false, 12> : (const void*)k_sweep_l128<false, 8>;
+}
+
 // Tables above the default 48 KB need the kernel's opt-in, once per device
 // (set at the first launch, which pa_init makes outside any stream capture).
 static cudaError_t ensure_smem_optin() {
@@ -1011,8 +1029,8 @@ static cudaError_t ensure_smem_optin() {
     if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
     const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
     const int t3max = (int)l64_plain_smem(true, L64_T3_MAX);
-    if ((e = cudaFuncSetAttribute(k_sweep_l64<false, true>, A, t3max)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_sweep_l64<true, true>, A, t3max)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(plain64(false, true), A, t3max)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(plain64(true, true), A, t3max)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_sweep_l64_batched<false>, A, (int)L64_BATCHED_SMEM)) !=
         cudaSuccess)
         return e;
@@ -1045,34 +1063,53 @@ static const void* pick(const RunDev& d, K64 f64f, K64 f64j, K128 f128f, K128 f1
     return pmj ? (const void*)f64j : (const void*)f64f;
 }
 
+// One block per SM (the register budget of its warps).
+static int sm_count() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    return sms;
+}
+
 int l64_grid(const RunDev& d) {
-    const int w = l64_block_warps(d);
-    // one CTA per SM in either form (the register budget of 12 warps)
-    const int full = wave(pick(d, k_sweep_l64<false, false>, k_sweep_l64<true, false>,
-                               k_sweep_l128<false>, k_sweep_l128<true>),
-                          w * 32, is_l128(d) ? 0 : l64_plain_smem(false, 0));
-    if (full <= 0) return 0;
-    const int64_t need = ((int64_t)d.cap + w - 1) / w;
-    return (int)(need < full ? need : full);
+    if (ensure_smem_optin() != cudaSuccess) return 0;
+    const int sms = sm_count();
+    return (int)((int64_t)d.cap < sms ? (int64_t)d.cap : sms);
+}
+
+// Warps per block of the L = 128 ferromagnet for `n` replicas: 8 or 12.  Every
+// warp takes one replica per round, and a round lasts 106, 131 or 205 us (theta =
+// 10, GB300) with 1, 2 or 3 warps per scheduler: 8 warps have the better rate, 12
+// fewer rounds where the last one of 8 would be nearly empty.  Measured, us per
+// launch with 8 / 12 warps: 1300 replicas 236 / 197, 2432 298 / 314, 5001 627 / 614,
+// 16384 1798 / 1838, 2^17 14106 / 14750.
+static int warps128_for(int64_t n, int sms) {
+    const int64_t t[4] = {0, 106, 131, 205};
+    auto cost = [&](int64_t k) {  // k warps per scheduler, 4 schedulers per SM
+        const int64_t slots = 4 * k * sms, rest = n % slots;
+        return n / slots * t[k] + t[(rest + 4 * sms - 1) / (4 * sms)];
+    };
+    return cost(3) < cost(2) ? 12 : 8;
 }
 
 cudaError_t launch_sweep_l64(const RunDev& d, int nsweeps, int grid, cudaStream_t s) {
     const cudaError_t e = ensure_smem_optin();
     if (e != cudaSuccess) return e;
     const bool pmj = d.model == PA_MODEL_PMJ;
+    RunDev dd = d;
+    int n = nsweeps;
+    void* args[] = {&dd, &n};
     if (is_l128(d)) {
-        if (pmj) k_sweep_l128<true><<<grid, warps128<true>() * 32, 0, s>>>(d, nsweeps);
-        else k_sweep_l128<false><<<grid, warps128<false>() * 32, 0, s>>>(d, nsweeps);
-    } else if (nsweeps >= 1 && nsweeps <= L64_T3_MAX) {
-        const size_t sm = l64_plain_smem(true, nsweeps);
-        if (pmj) k_sweep_l64<true, true><<<grid, WARPS64 * 32, sm, s>>>(d, nsweeps);
-        else k_sweep_l64<false, true><<<grid, WARPS64 * 32, sm, s>>>(d, nsweeps);
-    } else {
-        const size_t sm = l64_plain_smem(false, nsweeps);
-        if (pmj) k_sweep_l64<true, false><<<grid, WARPS64 * 32, sm, s>>>(d, nsweeps);
-        else k_sweep_l64<false, false><<<grid, WARPS64 * 32, sm, s>>>(d, nsweeps);
+        // the population fluctuates about R0; a streamed step sweeps a range of it
+        int64_t reps = (int64_t)d.R0 + (int64_t)std::sqrt((double)d.R0);
+        if (reps > (int64_t)d.slot_hi - d.slot_lo) reps = (int64_t)d.slot_hi - d.slot_lo;
+        const int w = pmj ? warps128<true>() : warps128_for(reps, grid);
+        return cudaLaunchKernel(plain128(pmj, w), dim3(grid), dim3(w * 32), args, 0, s);
     }
-    return cudaGetLastError();
+    const bool t3 = nsweeps >= 1 && nsweeps <= L64_T3_MAX;
+    return cudaLaunchKernel(plain64(pmj, t3), dim3(grid),
+                            dim3((pmj ? WARPS64_PMJ : WARPS64_FERRO) * 32), args,
+                            l64_plain_smem(t3, nsweeps), s);
 }
 
 // One block per SM.

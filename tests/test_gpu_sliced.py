@@ -70,3 +70,12 @@ def test_batched_classes_in_every_shape(P, warps):
             assert o.step() == 0
             compare_state(P, r, o, i)
     batch.close()
+
+
+@pytest.mark.parametrize("L,model,R0", [(64, 0, 151), (64, 0, 153), (64, 0, 16 * 152 + 1),
+                                        (64, 1, 12 * 152 + 1), (128, 0, 151), (128, 0, 8 * 152 + 3),
+                                        (128, 0, 12 * 152 - 60), (128, 1, 8 * 152 + 1)])
+def test_register_kernels_around_a_round(P, L, model, R0):
+    """Replicas dealt to the SMs one by one, in one round or a little more, and
+    both block sizes of the L = 128 ferromagnet."""
+    run_lockstep(P, steps=1, R0=R0, K=20, theta=1, **spec(2, L, 1, model))
