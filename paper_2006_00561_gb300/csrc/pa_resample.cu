@@ -209,6 +209,7 @@ __device__ __forceinline__ bool tau_run(const RunDev& d, uint32_t blk, uint32_t 
 }
 
 __global__ void __launch_bounds__(256) k_tau(__grid_constant__ const RunDev d) {
+    chain_wait();
     tau_run(d, blockIdx.x, gridDim.x);
 }
 
@@ -311,6 +312,7 @@ __device__ __forceinline__ void poisson_counts(const RunDev& d, uint32_t first, 
 }
 
 __global__ void __launch_bounds__(256) k_poisson_counts(__grid_constant__ const RunDev d) {
+    chain_wait();
     if (!d.st->active) return;
     poisson_counts(d, blockIdx.x * 256u + threadIdx.x, gridDim.x * 256u, d.st->R_prev);
 }
@@ -557,8 +559,15 @@ __device__ __forceinline__ void resample_tile(const RunDev& d, uint32_t tile, ui
 #define PA_RS_MINB 4
 #endif
 template <int RULE, bool SPLIT>
-__global__ void __launch_bounds__(RS_THREADS, PA_RS_MINB) k_resample(RunDev d) {
+__global__ void __launch_bounds__(RS_THREADS, PA_RS_MINB) k_resample(__grid_constant__ const RunDev d) {
     __shared__ ResampleSmem sm;
+    chain_wait();
+    if (d.clear_hist) {  // the reweight was their last reader
+        uint32_t* acc = reinterpret_cast<uint32_t*>(d.accum);  // accum, then the histogram
+        for (uint32_t k = blockIdx.x * RS_THREADS + threadIdx.x; k < 4u + (uint32_t)d.bins;
+             k += gridDim.x * RS_THREADS)
+            acc[k] = 0u;
+    }
     if (!d.st->active) return;
     const uint32_t R = d.st->R_prev;
     for (;;) {
@@ -816,7 +825,10 @@ __device__ __forceinline__ void obs_run(const RunDev& d, int nsweeps) {
     }
 }
 
-__global__ void __launch_bounds__(256) k_obs(__grid_constant__ const RunDev d, int nsweeps) { obs_run(d, nsweeps); }
+__global__ void __launch_bounds__(256) k_obs(__grid_constant__ const RunDev d, int nsweeps) {
+    chain_wait();
+    obs_run(d, nsweeps);
+}
 
 __global__ void __launch_bounds__(256) k_obs_batched(BatchDev b) {
 #if PA_RS_STAGE
@@ -833,8 +845,9 @@ __global__ void __launch_bounds__(256) k_obs_batched(BatchDev b) {
 }  // namespace
 
 cudaError_t launch_tau(const RunDev& d, cudaStream_t s) {
-    k_tau<<<tau_ctas(d.bins), 256, 0, s>>>(d);
-    return cudaGetLastError();
+    RunDev dd = d;
+    void* args[] = {&dd};
+    return launch_chained((const void*)k_tau, dim3(tau_ctas(d.bins)), dim3(256), 0, s, args);
 }
 
 // One wave of resident CTAs (capped by the number of tiles), looked up once
@@ -897,26 +910,21 @@ static int flat_grid(uint64_t n) {
 
 template <bool SPLIT>
 static cudaError_t launch_counts_scan(const RunDev& d, cudaStream_t s) {
+    RunDev dd = d;
+    void* args[] = {&dd};
     if (d.resample == PA_RESAMPLE_POISSON) {
         const int g = flat_grid(d.cap);
         if (g <= 0) return cudaErrorInvalidValue;
-        k_poisson_counts<<<g, 256, 0, s>>>(d);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_chained((const void*)k_poisson_counts, dim3(g), dim3(256), 0, s, args);
         if (e != cudaSuccess) return e;
     }
+    const bool drawn = d.resample != PA_RESAMPLE_NEAREST;
+    const void* fn = drawn ? (const void*)k_resample<2, SPLIT> : (const void*)k_resample<0, SPLIT>;
     // cache slots: 0 and 4 the one-kernel forms, 7 and 9 the split forms
-    if (d.resample != PA_RESAMPLE_NEAREST) {
-        const int grid = resample_wave((const void*)k_resample<2, SPLIT>, SPLIT ? 9 : 4,
-                                       d.tiles << d.slice_lg);
-        if (grid <= 0) return cudaErrorInvalidValue;
-        k_resample<2, SPLIT><<<grid, RS_THREADS, 0, s>>>(d);
-    } else {
-        const int grid = resample_wave((const void*)k_resample<0, SPLIT>, SPLIT ? 7 : 0,
-                                       d.tiles << d.slice_lg);
-        if (grid <= 0) return cudaErrorInvalidValue;
-        k_resample<0, SPLIT><<<grid, RS_THREADS, 0, s>>>(d);
-    }
-    return cudaGetLastError();
+    const int grid = resample_wave(fn, SPLIT ? (drawn ? 9 : 7) : (drawn ? 4 : 0),
+                                   d.tiles << d.slice_lg);
+    if (grid <= 0) return cudaErrorInvalidValue;
+    return launch_chained(fn, dim3(grid), dim3(RS_THREADS), 0, s, args);
 }
 
 cudaError_t launch_resample(const RunDev& d, cudaStream_t s) {
@@ -969,8 +977,9 @@ __device__ __forceinline__ unsigned long long block_sum_u64(unsigned long long v
     return tot;
 }
 
-__global__ void __launch_bounds__(RS_THREADS) k_mn_tile_sums(RunDev d) {
+__global__ void __launch_bounds__(RS_THREADS) k_mn_tile_sums(__grid_constant__ const RunDev d) {
     __shared__ unsigned long long sw[RS_THREADS / 32];
+    chain_wait();
     const DevState* st = d.st;
     if (!st->active) return;
     const uint32_t R = st->R_prev, src = st->src;
@@ -988,8 +997,9 @@ __global__ void __launch_bounds__(RS_THREADS) k_mn_tile_sums(RunDev d) {
 }
 
 // Exclusive scan of the tile sums in place; mn_tiles[ntiles] = the total.
-__global__ void __launch_bounds__(1024) k_mn_scan(RunDev d) {
+__global__ void __launch_bounds__(1024) k_mn_scan(__grid_constant__ const RunDev d) {
     __shared__ unsigned long long s[1024];
+    chain_wait();
     const DevState* st = d.st;
     if (!st->active) return;
     const uint32_t R = st->R_prev;
@@ -1017,8 +1027,9 @@ __global__ void __launch_bounds__(1024) k_mn_scan(RunDev d) {
 }
 
 // C_i per replica (inclusive), and the copy counts cleared for the draws.
-__global__ void __launch_bounds__(RS_THREADS) k_mn_cum(RunDev d) {
+__global__ void __launch_bounds__(RS_THREADS) k_mn_cum(__grid_constant__ const RunDev d) {
     __shared__ unsigned long long sw[RS_THREADS / 32];
+    chain_wait();
     const DevState* st = d.st;
     if (!st->active) return;
     const uint32_t R = st->R_prev, src = st->src;
@@ -1056,7 +1067,8 @@ __global__ void __launch_bounds__(RS_THREADS) k_mn_cum(RunDev d) {
     }
 }
 
-__global__ void __launch_bounds__(256) k_mn_draw(RunDev d) {
+__global__ void __launch_bounds__(256) k_mn_draw(__grid_constant__ const RunDev d) {
+    chain_wait();
     const DevState* st = d.st;
     if (!st->active) return;
     const uint32_t R = st->R_prev, step = st->step;
@@ -1091,18 +1103,28 @@ cudaError_t launch_multinomial(const RunDev& d, cudaStream_t s) {
     if (!d.mn_cum || !d.mn_tiles) return cudaErrorInvalidValue;
     const int wave = resample_wave((const void*)k_mn_cum, 5, d.tiles);
     if (wave <= 0) return cudaErrorInvalidValue;
-    k_mn_tile_sums<<<wave, RS_THREADS, 0, s>>>(d);
-    k_mn_scan<<<1, 1024, 0, s>>>(d);
-    k_mn_cum<<<wave, RS_THREADS, 0, s>>>(d);
     const int g = flat_grid((d.R0 + 1u) / 2u);
     if (g <= 0) return cudaErrorInvalidValue;
-    k_mn_draw<<<g, 256, 0, s>>>(d);
-    return cudaGetLastError();
+    RunDev dd = d;
+    void* args[] = {&dd};
+    const struct {
+        const void* fn;
+        int grid, threads;
+    } pass[] = {{(const void*)k_mn_tile_sums, wave, RS_THREADS},
+                {(const void*)k_mn_scan, 1, 1024},
+                {(const void*)k_mn_cum, wave, RS_THREADS},
+                {(const void*)k_mn_draw, g, 256}};
+    for (const auto& p : pass) {
+        const cudaError_t e = launch_chained(p.fn, dim3(p.grid), dim3(p.threads), 0, s, args);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_obs(const RunDev& d, int nsweeps, cudaStream_t s) {
-    k_obs<<<1, 256, 0, s>>>(d, nsweeps);
-    return cudaGetLastError();
+    RunDev dd = d;
+    void* args[] = {&dd, &nsweeps};
+    return launch_chained((const void*)k_obs, dim3(1), dim3(256), 0, s, args);
 }
 
 cudaError_t launch_tau_batched(const BatchDev& b, cudaStream_t s) {

@@ -644,6 +644,7 @@ __global__ void __launch_bounds__(Team<DIM, L, RSP>::TT)
     uint32_t* sums = reinterpret_cast<uint32_t*>(smem + 64);
     uint32_t* S = reinterpret_cast<uint32_t*>(smem + 80);
     uint8_t* JS = reinterpret_cast<uint8_t*>(smem + 80 + s_quads<DIM, L>());
+    chain_wait();
     if constexpr (PMJ) couplings<DIM, L>(d, JS, threadIdx.x, Team<DIM, L, RSP>::TT);
     const SweepCtx x = sweep_ctx(d);
     const Keys K{d.rk0, d.rk1};
@@ -979,7 +980,7 @@ cudaError_t launch_sweep(const RunDev& d, int nsweeps, int grid, cudaStream_t s)
     RunDev dd = d;
     int n = nsweeps;
     void* args[] = {&dd, &n};
-    return cudaLaunchKernel(k.fn, dim3(grid), dim3(k.threads), args, (size_t)k.smem, s);
+    return launch_chained(k.fn, dim3(grid), dim3(k.threads), (size_t)k.smem, s, args);
 }
 
 bool batched_warps_valid(const RunDev& proto, int warps) {

@@ -538,6 +538,7 @@ __device__ __forceinline__ void cta_tables(uint2* tab, uint32_t ctag, uint32_t g
 template <bool PMJ, bool T3, int W>
 __global__ void __launch_bounds__(W * 32, 1)
     k_sweep_l64(__grid_constant__ const RunDev d, int nsweeps) {
+    chain_wait();
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     DevState* st = d.st;
     const uint32_t R = st->R;
@@ -834,6 +835,7 @@ __device__ __forceinline__ uint32_t l128_replica(const Keys& K, uint4* spins, ui
 template <bool PMJ, int W>
 __global__ void __launch_bounds__(W * 32, 1)
     k_sweep_l128(__grid_constant__ const RunDev d, int nsweeps) {
+    chain_wait();
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     DevState* st = d.st;
     const uint32_t R = st->R;
@@ -1104,12 +1106,11 @@ cudaError_t launch_sweep_l64(const RunDev& d, int nsweeps, int grid, cudaStream_
         int64_t reps = (int64_t)d.R0 + (int64_t)std::sqrt((double)d.R0);
         if (reps > (int64_t)d.slot_hi - d.slot_lo) reps = (int64_t)d.slot_hi - d.slot_lo;
         const int w = pmj ? warps128<true>() : warps128_for(reps, grid);
-        return cudaLaunchKernel(plain128(pmj, w), dim3(grid), dim3(w * 32), args, 0, s);
+        return launch_chained(plain128(pmj, w), dim3(grid), dim3(w * 32), 0, s, args);
     }
     const bool t3 = nsweeps >= 1 && nsweeps <= L64_T3_MAX;
-    return cudaLaunchKernel(plain64(pmj, t3), dim3(grid),
-                            dim3((pmj ? WARPS64_PMJ : WARPS64_FERRO) * 32), args,
-                            l64_plain_smem(t3, nsweeps), s);
+    return launch_chained(plain64(pmj, t3), dim3(grid), dim3((pmj ? WARPS64_PMJ : WARPS64_FERRO) * 32),
+                          l64_plain_smem(t3, nsweeps), s, args);
 }
 
 // One block per SM.
