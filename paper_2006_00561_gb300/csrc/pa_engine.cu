@@ -478,7 +478,7 @@ int pa_init(const pa_config* cfg, void* ws, size_t bytes, void* stream, pa_run**
     d.cap_alloc = (uint32_t)l.cap;
     d.R0 = (uint32_t)cfg->R0;
     d.tiles = (uint32_t)l.tiles;
-    d.slice_lg = pa::resample_slices((uint64_t)l.tiles);
+    d.slice_lg = pa::resample_slices((uint64_t)l.stride, (uint64_t)l.cap * l.stride, 1u << 14);
     d.mn_cum = l.mn_cum ? (unsigned long long*)(base + l.mn_cum) : nullptr;
     d.mn_tiles = l.mn_tiles ? (unsigned long long*)(base + l.mn_tiles) : nullptr;
     r->hist_bytes = 16 + (size_t)l.bins * 4;
@@ -1341,7 +1341,7 @@ int batch_init(pa_run* const* runs, int32_t nruns, const int32_t* steps_left, vo
     for (double& m : b->prof_ms) m = 0.0;
     std::vector<pa::RunDev> h_runs;
     std::vector<uint32_t> tile_base(1, 0u);
-    uint64_t tiles = 0;
+    uint64_t bytes_all = 0;
     for (int32_t i = 0; i < nruns; ++i) {
         pa_run* r = runs[i];
         if (!r || r->gather_pending) {
@@ -1371,13 +1371,12 @@ int batch_init(pa_run* const* runs, int32_t nruns, const int32_t* steps_left, vo
         if (left < b->steps_left) b->steps_left = left;
         b->runs.push_back(r);
         h_runs.push_back(r->d);
-        tiles += r->d.tiles;
+        bytes_all += (uint64_t)r->d.cap * r->d.stride;
     }
-    // one launch resamples all runs: slices by the tiles of the whole batch
-    const uint32_t slice_lg = pa::resample_slices(tiles);
+    // one launch resamples all runs: slices by the bytes of the whole batch
     for (auto& d : h_runs) {
-        d.slice_lg = slice_lg;
-        tile_base.push_back(tile_base.back() + (d.tiles << slice_lg));
+        d.slice_lg = pa::resample_slices(d.stride, bytes_all, 1u << 16);
+        tile_base.push_back(tile_base.back() + (d.tiles << d.slice_lg));
     }
     const int sliced_warps = pa::batched_default_warps(h_runs.data(), nruns);
     // classes: one sweep kernel instantiation per (layout, dim, L, model)
@@ -1441,7 +1440,6 @@ int batch_init(pa_run* const* runs, int32_t nruns, const int32_t* steps_left, vo
     b->bd.nruns = (uint32_t)nruns;
     b->bd.tile_base = d_tile_base;
     b->bd.total_tiles = tile_base.back();
-    b->bd.slice_lg = slice_lg;
     b->bd.max_bins = 1;
     for (const auto& h : h_runs)
         if (h.bins > b->bd.max_bins) b->bd.max_bins = h.bins;

@@ -118,7 +118,6 @@ struct BatchDev {
     int64_t max_bins;            // energy levels of the run with the most
     const uint32_t* tile_base;   // [nruns + 1] prefix sums of each run's slices of tiles
     uint32_t total_tiles;        // slices of all tiles
-    uint32_t slice_lg;           // log2 of the slices of a tile (every run's RunDev::slice_lg)
     uint32_t any_poisson;        // some run resamples by the Poisson rule
     uint32_t any_multinomial;    // some run resamples by multinomial draws
     uint32_t* counters;          // [0]: resample tiles, [1 + c]: sweep chunks of class c
@@ -336,17 +335,19 @@ int l64_batched_grid(const RunDev& proto);
 constexpr int RS_THREADS = 256;
 constexpr int RS_ITEMS = PA_RS_ITEMS;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
-// log2 of the slices of a tile for `tiles` tiles that one launch resamples.
-// One CTA gathers at about 30 GB/s whatever else runs, so the launch needs as
-// many CTAs as the GPU holds (152 x 4); a population of fewer tiles has
-// several CTAs count the whole of a tile (a microsecond or two) and each
-// gather its slice, of at least 32 replicas.
-#ifndef PA_RS_SPREAD
-#define PA_RS_SPREAD 608
-#endif
-inline uint32_t resample_slices(uint64_t tiles) {
+// log2 of the slices of a run's tiles, in a launch that resamples `total` bytes
+// of spins.  One CTA gathers at about 30 GB/s whatever else runs, so the launch
+// needs its bytes spread over as many CTAs as the GPU holds (152 x 4); where
+// there are fewer tiles, or tiles of more bytes than that, several CTAs count the
+// whole of a tile (a microsecond or two) and each gather its slice, of at least
+// 32 replicas and `least` bytes.  In a batch the bytes matter, not the tiles: with one
+// slice width for all, a tile of L = 128 (2 KB per replica) held the launch up.
+constexpr uint32_t RS_CTAS = 608;
+inline uint32_t resample_slices(uint64_t stride, uint64_t total, uint64_t least) {
+    uint64_t target = total / RS_CTAS;
+    if (target < least) target = least;
     uint32_t lg = 0;
-    while ((RS_TILE >> (lg + 1)) >= 32 && (tiles << (lg + 1)) <= PA_RS_SPREAD) ++lg;
+    while (((uint32_t)RS_TILE >> (lg + 1)) >= 32 && ((uint64_t)RS_TILE >> lg) * stride > target) ++lg;
     return lg;
 }
 

@@ -317,10 +317,10 @@ __global__ void __launch_bounds__(256) k_poisson_counts(__grid_constant__ const 
     poisson_counts(d, blockIdx.x * 256u + threadIdx.x, gridDim.x * 256u, d.st->R_prev);
 }
 
-// Batched: CTA g takes resample tile g of the batch, if its run is on the rule.
+// Batched: CTA g takes slice g of the batch, if its run is on the rule.
 __global__ void __launch_bounds__(RS_THREADS) k_poisson_counts_batched(BatchDev b) {
     __shared__ RunDev s_d;
-    const uint32_t g = blockIdx.x << b.slice_lg;
+    const uint32_t g = blockIdx.x;
     uint32_t lo = 0, hi = b.nruns;  // tile_base[lo] <= g < tile_base[hi]
     while (hi - lo > 1) {
         const uint32_t mid = (lo + hi) >> 1;
@@ -330,10 +330,9 @@ __global__ void __launch_bounds__(RS_THREADS) k_poisson_counts_batched(BatchDev 
     if (b.runs[lo].resample != PA_RESAMPLE_POISSON || !b.runs[lo].st->active) return;
     stage_run(&b.runs[lo], s_d);
     __syncthreads();
-    const uint32_t base = ((g - b.tile_base[lo]) >> b.slice_lg) * (uint32_t)RS_TILE;
-    const uint32_t R = s_d.st->R_prev;
-    if (base < R)
-        poisson_counts(s_d, base + threadIdx.x, RS_THREADS, min(R, base + (uint32_t)RS_TILE));
+    const uint32_t width = (uint32_t)RS_TILE >> s_d.slice_lg;
+    const uint32_t base = (g - b.tile_base[lo]) * width, R = s_d.st->R_prev;
+    if (base < R) poisson_counts(s_d, base + threadIdx.x, RS_THREADS, min(R, base + width));
 }
 
 // RULE 0 compiles the nearest-integer rule alone (the register budget of the
@@ -1134,7 +1133,7 @@ cudaError_t launch_tau_batched(const BatchDev& b, cudaStream_t s) {
 
 cudaError_t launch_resample_batched(const BatchDev& b, cudaStream_t s) {
     if (b.any_poisson) {
-        k_poisson_counts_batched<<<b.total_tiles >> b.slice_lg, RS_THREADS, 0, s>>>(b);
+        k_poisson_counts_batched<<<b.total_tiles, RS_THREADS, 0, s>>>(b);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

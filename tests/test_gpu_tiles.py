@@ -14,7 +14,7 @@ from oracle import oracle as O
 
 pytestmark = pytest.mark.gpu
 
-TILE, SPREAD = 2048, 608  # a tile is shared by as many CTAs as keep a launch within SPREAD
+TILE, SPREAD = 2048, 608  # tiles that fill the GPU with one CTA each
 
 
 @pytest.fixture(scope="module")
