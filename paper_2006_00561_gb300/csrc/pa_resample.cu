@@ -41,24 +41,32 @@ __device__ __forceinline__ void stage_run(const RunDev* src, RunDev& dst) {
 }
 
 // Calls f(k, H_k) for the occupied levels of the thread's share of the
-// histogram (four consecutive levels of every 4 * 256).
+// histogram (four consecutive levels of every 4 * 256), eight 16-byte loads at a
+// time before their conditions.
 template <typename F>
 __device__ __forceinline__ void each_level(const uint32_t* hist, uint32_t bins, F&& f) {
     const uint4* h4 = reinterpret_cast<const uint4*>(hist);  // 16-byte aligned
     const uint32_t quads = bins >> 2;
-#pragma unroll 4
-    for (uint32_t q = threadIdx.x; q < quads; q += 256) {
-        const uint4 h = h4[q];
-        if (h.x) f(4 * q, h.x);
-        if (h.y) f(4 * q + 1, h.y);
-        if (h.z) f(4 * q + 2, h.z);
-        if (h.w) f(4 * q + 3, h.w);
+    const uint32_t kt = 4 * quads + threadIdx.x;
+    const uint32_t tail = kt < bins ? hist[kt] : 0u;
+    for (uint32_t q0 = threadIdx.x; q0 < quads; q0 += 8 * 256) {
+        uint4 h[8];
+#pragma unroll
+        for (uint32_t j = 0; j < 8; ++j) {
+            const uint32_t q = q0 + 256 * j;
+            h[j] = q < quads ? h4[q] : make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (uint32_t j = 0; j < 8; ++j) {
+            if ((h[j].x | h[j].y | h[j].z | h[j].w) == 0u) continue;
+            const uint32_t k = 4 * (q0 + 256 * j);
+            if (h[j].x) f(k, h[j].x);
+            if (h[j].y) f(k + 1, h[j].y);
+            if (h[j].z) f(k + 2, h[j].z);
+            if (h[j].w) f(k + 3, h[j].w);
+        }
     }
-    const uint32_t k = 4 * quads + threadIdx.x;
-    if (k < bins) {
-        const uint32_t h = hist[k];
-        if (h) f(k, h);
-    }
+    if (tail) f(kt, tail);
 }
 
 // Reweight of one run by nblk 256-thread CTAs.  Every CTA finds kref and S
@@ -67,14 +75,38 @@ __device__ __forceinline__ void each_level(const uint32_t* hist, uint32_t bins, 
 // the step index and R, advances the run's scalars.  Returns whether this CTA
 // is the one that was last to read the histogram.
 //
-// Bound: GB300 retires about two FP64 operations per SM and clock, so the
-// latency is the FP64 work of one CTA.  Hence levels without replicas add
-// nothing (x + 0 * D is x, exactly) and are skipped, levels whose tau is below
-// 2^-33 get (0, 0) without a division, more CTAs share the divisions, and the
-// two logarithms run in a warp of their own beside them.  Before -> after, timed
-// by events: 13.4 -> 12.2 us (257 levels), 25 -> 14.7 (4097), 44 -> 24 (16385); a
-// batch of 28 runs with up to 16385 levels 87 -> 39.
+// Bound: an FP64 operation takes some 140 cycles on GB300 and a division 1450, so
+// the time is the chain of FP64 operations.  Hence the products H_k D are
+// formed by all threads ahead of the chunks' sums, levels without replicas add
+// nothing (x + 0 * D is x, exactly) and are skipped, one warp alone adds up the
+// chunk sums, levels whose tau is below 2^-33 get (0, 0) without a division, n and
+// F are cut from the bits of tau, and the logarithms run in a warp of their own
+// beside the divisions.  us, timed by events around the launch, with FP64 work on
+// every level -> so: 13.4 -> 10.3 (257 levels), 25 -> 12.2 (4097), 44 -> 17 (16385); a batch
+// of 28 runs with up to 16385 levels 87 -> 24.
 constexpr uint32_t TAU_LEVELS = 128;  // levels per CTA and pass
+// Levels whose products a CTA holds at a time (any more are added in further
+// passes over the occupied range).
+constexpr uint32_t TAU_HELD = 2048;
+
+// floor(x) and floor(2^32 frac(x)) of x >= 0 (exact: both are bits of x);
+// floor saturates at 2^32 - 1.
+__device__ __forceinline__ void split32(double x, uint32_t& n, uint32_t& F) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+    const int e = (int)(bits >> 52) - 1023;  // x >= 0: no sign
+    const unsigned long long m = (bits & 0xfffffffffffffull) | 0x10000000000000ull;  // x = m 2^(e - 52)
+    n = F = 0;
+    if (e >= 32) {
+        if (e == 1024 && m != 0x10000000000000ull) return;  // not a number: (0, 0)
+        n = 0xffffffffu;
+        if (e < 52) F = (uint32_t)(((m << (e + 12)) >> 32));
+    } else if (e >= 0) {
+        n = (uint32_t)(m >> (52 - e));
+        F = (uint32_t)((m << (e + 12)) >> 32);
+    } else if (e >= -32) {
+        F = (uint32_t)(m >> (20 - e));
+    }
+}
 // CTAs of a run at most: 33, 65 and 130 run alike on GB300 (14.7 us at 4097
 // levels, 24 us at 16385, timed by events around the launch).
 #ifndef PA_TAU_CTAS
@@ -83,13 +115,15 @@ constexpr uint32_t TAU_LEVELS = 128;  // levels per CTA and pass
 constexpr uint32_t TAU_CTAS = PA_TAU_CTAS;
 __device__ __forceinline__ bool tau_run(const RunDev& d, uint32_t blk, uint32_t nblk) {
     DevState* st = d.st;
+    __shared__ double s_prod[TAU_HELD];
     __shared__ double s_part[8];
-    __shared__ double s_lnR;
+    __shared__ double s_S;
     __shared__ uint32_t s_min[8], s_max[8];
     __shared__ unsigned long long s_sum;
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const uint32_t i = st->step + 1;
-    const uint32_t R = st->R;
+    const uint32_t R = st->R, cur = st->cur, epoch = st->epoch, negbonds = st->negbonds;
+    const double lnZ = st->lnZ;
     const uint32_t bins = (uint32_t)d.bins;
     if (i > (uint32_t)d.K || R == 0) {
         if (t == 0 && blk == 0) {
@@ -116,8 +150,6 @@ __device__ __forceinline__ bool tau_run(const RunDev& d, uint32_t blk, uint32_t 
         s_min[wid] = kmin;
         s_max[wid] = kmax;
     }
-    const bool logs = blk == nblk - 1;  // this CTA also takes ln Q and the check of sum H
-    if (logs && t == 160) s_lnR = log((double)R);
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < 8; ++w) {
@@ -125,63 +157,67 @@ __device__ __forceinline__ bool tau_run(const RunDev& d, uint32_t blk, uint32_t 
         kmax = max(kmax, s_max[w]);
     }
     const uint32_t kref = heating ? kmax : kmin;
+    const bool logs = blk == nblk - 1;  // this CTA also takes ln Q and the check of sum H
     if (logs && hs) atomicAdd(&s_sum, hs);
     // S in the fixed order: 256 contiguous chunks summed left to right, then a
     // pairwise tree over the chunk sums; level k weighs D[|k - kref|].
     const uint32_t ch = (bins + 255) / 256;
     const uint32_t k_lo = max(t * ch, kmin), k_hi = min(min((t + 1) * ch, bins), kmax + 1u);
     double acc = 0.0;
-    for (uint32_t k0 = k_lo; k0 < k_hi; k0 += 8) {
-        uint32_t h[8];
-        double w[8];
-#pragma unroll
-        for (uint32_t j = 0; j < 8; ++j) {
-            const uint32_t k = k0 + j;
-            h[j] = 0;
-            if (k < k_hi) {
-                h[j] = d.hist[k];
-                w[j] = D[heating ? kref - k : k - kref];
-            }
+    for (uint32_t b0 = kmin; b0 <= kmax; b0 += TAU_HELD) {  // kmin > kmax: no replicas
+        const uint32_t b1 = min(b0 + TAU_HELD, kmax + 1u);
+        for (uint32_t k = b0 + t; k < b1; k += 256) {
+            const uint32_t h = d.hist[k];
+            s_prod[k - b0] = h ? __dmul_rn((double)h, D[heating ? kref - k : k - kref]) : -1.0;
         }
-#pragma unroll
-        for (uint32_t j = 0; j < 8; ++j)
-            if (h[j]) acc = __dadd_rn(acc, __dmul_rn((double)h[j], w[j]));
+        __syncthreads();
+        const uint32_t lo = max(k_lo, b0), hi = min(k_hi, b1);
+        for (uint32_t k = lo; k < hi; ++k) {
+            const double p = s_prod[k - b0];
+            if (__double_as_longlong(p) >= 0) acc = __dadd_rn(acc, p);
+        }
+        __syncthreads();
     }
-    if (__any_sync(0xffffffffu, acc != 0.0)) {
+    if (__any_sync(0xffffffffu, __double_as_longlong(acc) != 0)) {
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) acc = __dadd_rn(acc, __shfl_xor_sync(0xffffffffu, acc, o));
     }
     if (lane == 0) s_part[wid] = acc;
     __syncthreads();
-    const double S = __dadd_rn(
-        __dadd_rn(__dadd_rn(s_part[0], s_part[1]), __dadd_rn(s_part[2], s_part[3])),
-        __dadd_rn(__dadd_rn(s_part[4], s_part[5]), __dadd_rn(s_part[6], s_part[7])));
+    if (wid == 0) {
+        double v = s_part[lane & 7];
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+        if (lane == 0) s_S = v;
+    }
+    __syncthreads();
+    const double S = s_S;
     if (wid < 4) {
         const double R0d = (double)d.R0;
-        const double least = __dmul_rn(S, 5.8207660913467407e-11);  // 2^-34 S: tau < 2^-33
+        const long long least =  // 2^-34 S: tau < 2^-33 (positive doubles order like their bits)
+            __double_as_longlong(__dmul_rn(S, 5.8207660913467407e-11));
         for (uint32_t k = blk * TAU_LEVELS + t; k < bins; k += nblk * TAU_LEVELS) {
             uint32_t n = 0, F = 0;
             const int64_t j = heating ? (int64_t)kref - (int64_t)k : (int64_t)k - (int64_t)kref;
             if (j >= 0) {
                 const double w = __dmul_rn(R0d, D[j]);
-                if (!(w < least)) {
-                    const double tau = __ddiv_rn(w, S);
-                    const double nk = floor(tau);
-                    n = (uint32_t)nk;
-                    F = (uint32_t)floor(__dmul_rn(__dsub_rn(tau, nk), 4294967296.0));
-                }
+                if (__double_as_longlong(w) >= least) split32(__ddiv_rn(w, S), n, F);
             }
             d.tab_n[k] = n;
             d.tab_F[k] = F;
         }
-    } else if (logs && t == 128) {
-        if (s_sum != (unsigned long long)R) atomicOr(&st->status, ST_INVARIANT);
-        const long long parity = st->negbonds & 1u;
-        const long long Eref = 2 * (2 * (long long)kref + parity) - (long long)d.dim * d.N;
-        const double lnQ = __dsub_rn(__dsub_rn(log(S), s_lnR), __dmul_rn(db, (double)Eref));
-        st->lnQ = lnQ;
-        st->lnZ = __dadd_rn(st->lnZ, lnQ);
-        st->S = S;
+    } else if (logs && wid == 4) {
+        const double ln = log(lane == 1 ? (double)R : S);  // both logarithms at once
+        const double lnR = __shfl_sync(0xffffffffu, ln, 1);
+        if (lane == 0) {
+            if (s_sum != (unsigned long long)R) atomicOr(&st->status, ST_INVARIANT);
+            const long long Eref =
+                2 * (2 * (long long)kref + (long long)(negbonds & 1u)) - (long long)d.dim * d.N;
+            const double lnQ = __dsub_rn(__dsub_rn(ln, lnR), __dmul_rn(db, (double)Eref));
+            st->lnQ = lnQ;
+            st->lnZ = __dadd_rn(lnZ, lnQ);
+            st->S = S;
+        }
     }
     if (nblk > 1) {
         __shared__ bool s_last;
@@ -198,9 +234,8 @@ __device__ __forceinline__ bool tau_run(const RunDev& d, uint32_t blk, uint32_t 
         st->kref = kref;
         st->step = i;
         st->R_prev = R;
-        st->epoch = st->epoch + 1;
+        st->epoch = epoch + 1;
         st->tile_counter = 0;
-        const uint32_t cur = st->cur;
         st->src = cur;
         st->cur = cur ^ 1u;
         st->active = 1;
@@ -561,21 +596,27 @@ template <int RULE, bool SPLIT>
 __global__ void __launch_bounds__(RS_THREADS, PA_RS_MINB) k_resample(__grid_constant__ const RunDev d) {
     __shared__ ResampleSmem sm;
     chain_wait();
+    if (threadIdx.x == 0) sm.tile = atomicAdd(&d.st->tile_counter, 1u);
+    const bool active = d.st->active != 0;
+    const uint32_t R = d.st->R_prev;
     if (d.clear_hist) {  // the reweight was their last reader
         uint32_t* acc = reinterpret_cast<uint32_t*>(d.accum);  // accum, then the histogram
         for (uint32_t k = blockIdx.x * RS_THREADS + threadIdx.x; k < 4u + (uint32_t)d.bins;
              k += gridDim.x * RS_THREADS)
             acc[k] = 0u;
     }
-    if (!d.st->active) return;
-    const uint32_t R = d.st->R_prev;
+    if (!active) return;
+    // with a CTA for every slice each claims one and none has to look for more
+    const bool single = gridDim.x >= ((R + (uint32_t)RS_TILE - 1) / (uint32_t)RS_TILE) << d.slice_lg;
+    __syncthreads();
     for (;;) {
+        const uint32_t id = sm.tile, tile = id >> d.slice_lg;
+        if (tile >= (R + (uint32_t)RS_TILE - 1) / (uint32_t)RS_TILE) break;
+        resample_tile<RULE, SPLIT>(d, tile, id & ((1u << d.slice_lg) - 1u), sm);
+        if (single) break;
+        __syncthreads();  // sm is reused by the next tile
         if (threadIdx.x == 0) sm.tile = atomicAdd(&d.st->tile_counter, 1u);
         __syncthreads();
-        const uint32_t id = sm.tile, tile = id >> d.slice_lg;
-        if (tile * (uint32_t)RS_TILE >= R) break;
-        resample_tile<RULE, SPLIT>(d, tile, id & ((1u << d.slice_lg) - 1u), sm);
-        __syncthreads();  // sm is reused by the next tile
     }
 }
 
@@ -755,25 +796,29 @@ __device__ __forceinline__ long long warp_sum_ll(long long v) {
 }
 
 // The record of the measured step: integer sums over the histogram by the CTA,
-// then the averages, one per lane of a warp (an FP64 division is a chain of
-// some ten dependent FP64 operations: two of them one after the other instead
-// of eight; 10.0 -> 8.3 us at 4097 levels, timed by events).
+// then the averages, one per lane of a warp (an FP64 division takes some 1450
+// cycles on GB300: two of them one after the other instead of eight).  Loads
+// that depend on nothing come first.  us, timed by events: 10.0 -> 8.3 (4097
+// levels), 12.6 -> 8.3 (16385).
 __device__ __forceinline__ void obs_run(const RunDev& d, int nsweeps) {
     DevState* st = d.st;
     __shared__ long long s_part[3][8];
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    const uint32_t step = st->step, R = st->R;
-    const long long parity = st->negbonds & 1u;
+    const uint32_t step = st->step, R = st->R, negbonds = st->negbonds, base = st->sweep_base;
+    const unsigned long long done = st->sweeps_done;
+    const double lnQ = st->lnQ, lnZ = st->lnZ;
+    const long long mags = lane == 2 || lane == 3 ? (long long)d.accum[lane - 2] : 0ll;
     const long long dimN = (long long)d.dim * d.N;
-    const double beta = d.beta[step];
+    const long long E0 = 2 * (long long)(negbonds & 1u) - dimN;  // energy of level 0
     long long cnt = 0, sE = 0, sE2 = 0;
     each_level(d.hist, (uint32_t)d.bins, [&](uint32_t k, uint32_t h) {
-        const long long E = 2 * (2 * (long long)k + parity) - dimN;
+        const long long E = E0 + 4 * (long long)k;
         const long long hE = (long long)h * E;
         cnt += h;
         sE += hE;
         sE2 += hE * E;
     });
+    const double beta = d.beta[step];
     cnt = warp_sum_ll(cnt);
     sE = warp_sum_ll(sE);
     sE2 = warp_sum_ll(sE2);
@@ -792,21 +837,16 @@ __device__ __forceinline__ void obs_run(const RunDev& d, int nsweeps) {
         p2 += s_part[2][w];
     }
     // lanes 0..3: sum E, sum E^2, sum |M|, sum M^2 and their averages
-    const long long sum = lane == 0   ? p1
-                          : lane == 1 ? p2
-                          : lane < 4  ? (long long)d.accum[lane - 2]
-                                      : 0ll;
-    const double Nd = (double)d.N;
+    const long long sum = lane == 0 ? p1 : lane == 1 ? p2 : mags;
     const double mean = __ddiv_rn((double)sum, (double)R);
     const double mE = __shfl_sync(0xffffffffu, mean, 0), mE2 = __shfl_sync(0xffffffffu, mean, 1);
     const double mA = __shfl_sync(0xffffffffu, mean, 2), mM2 = __shfl_sync(0xffffffffu, mean, 3);
     // lanes 0..3: e, cv, m_abs, chi
-    const double num =
-        lane == 0   ? mE
-        : lane == 1 ? __dmul_rn(__dmul_rn(beta, beta), __dsub_rn(mE2, __dmul_rn(mE, mE)))
-        : lane == 2 ? mA
-                    : __dmul_rn(beta, __dsub_rn(mM2, __dmul_rn(mA, mA)));
-    const double avg = __ddiv_rn(num, Nd);
+    const double sq = lane == 1 ? mE : mA, sq2 = lane == 1 ? mE2 : mM2;
+    const double var = __dsub_rn(sq2, __dmul_rn(sq, sq));
+    const double fac = lane == 1 ? __dmul_rn(beta, beta) : beta;
+    const double num = lane == 0 ? mE : lane == 2 ? mA : __dmul_rn(fac, var);
+    const double avg = __ddiv_rn(num, (double)d.N);
     pa_obs* o = d.obs + step;
     if (lane < 4) {
         (&o->sumE)[lane] = sum;
@@ -817,10 +857,10 @@ __device__ __forceinline__ void obs_run(const RunDev& d, int nsweeps) {
         o->step = step;
         o->R = R;
         o->beta = beta;
-        o->lnQ = st->lnQ;
-        o->lnZ = st->lnZ;
-        st->sweep_base = st->sweep_base + (uint32_t)nsweeps;
-        st->sweeps_done = st->sweeps_done + (unsigned long long)nsweeps;
+        o->lnQ = lnQ;
+        o->lnZ = lnZ;
+        st->sweep_base = base + (uint32_t)nsweeps;
+        st->sweeps_done = done + (unsigned long long)nsweeps;
     }
 }
 
