@@ -1,5 +1,5 @@
-"""The replica-sliced sweep in both of its forms, every lattice and layout:
-populations around a chunk of 32 replicas, populations on both sides of the
+"""The replica-sliced sweep in all of its forms, every lattice and layout:
+populations around a chunk of replicas, populations on both sides of the
 line between four lanes per group and one, and batched classes in every block
 shape.  Bit for bit against the oracle."""
 from __future__ import annotations
@@ -45,6 +45,16 @@ def test_populations_around_the_line_between_the_forms(P, dim, L, layout, model,
     per_chunk = (L ** dim // 8 + 31) // 32
     chunks = -(-FOUR_BELOW // per_chunk)  # the fewest that take one lane per group
     R0 = 32 * (chunks - 1) + (1 if side > 0 else 0)
+    run_lockstep(P, steps=1, R0=R0, K=20, theta=1, **spec(dim, L, layout, model))
+
+
+@pytest.mark.parametrize("dim,L,layout,model,R0",
+                         [(2, 16, 0, 0, 4801), (2, 16, 1, 1, 9999), (2, 32, 0, 0, 1999),
+                          (2, 32, 1, 0, 4701), (3, 6, 1, 1, 4099), (3, 6, 0, 0, 7900),
+                          (3, 8, 1, 1, 2001), (3, 10, 0, 1, 2003), (3, 10, 1, 1, 4050),
+                          (3, 12, 1, 0, 1601), (2, 64, 0, 1, 1700)])
+def test_chunks_of_16_and_32_replicas(P, dim, L, layout, model, R0):
+    """Smaller populations take chunks of eight (test_small_populations)."""
     run_lockstep(P, steps=1, R0=R0, K=20, theta=1, **spec(dim, L, layout, model))
 
 
