@@ -569,8 +569,9 @@ __device__ __forceinline__ void team_chunk(const RunDev& d, const SweepCtx& x, u
     static_assert(RPQ == 8 || RSP == 4, "only four lanes per group take part of the chunk's bits");
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     // bit (and lane) 8 q + r is replica r of quarter q; r < RPQ
-    const uint32_t slot = b0 + (uint32_t)((lane >> 3) * RPQ + (lane & 7));
-    const bool valid = (lane & 7) < RPQ && slot < x.R, i8 = d.layout == PA_LAYOUT_INT8;
+    const uint32_t slot = b0 + (uint32_t)(RPQ == 8 ? lane : (lane >> 3) * RPQ + (lane & 7));
+    const bool valid = (RPQ == 8 || (lane & 7) < RPQ) && slot < x.R;
+    const bool i8 = d.layout == PA_LAYOUT_INT8;
     uint8_t* rep = d.spins[x.cur] + (size_t)slot * d.stride;
 #pragma unroll 1
     for (int u = wid; u < G::UNITS; u += TM::NW) load_unit<DIM, L>(rep, i8, d.stride, valid, S, u, lane);

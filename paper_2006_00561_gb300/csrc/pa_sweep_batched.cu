@@ -19,10 +19,22 @@ __device__ __forceinline__ uint32_t run_of(const BatchSweepArgs& a, uint32_t g, 
     return a.run_ids[lo];
 }
 
+// Blocks that the register budget leaves room for on an SM: with the round keys
+// in registers the compiler takes up to 128 of them, and the SM then holds half
+// the warps of the plain kernel.  us of a batched sweep on GB300 with room for 512,
+// 640, 768, 1024 threads: 24 spin glasses of three sizes 887, 851, 873, 883; 12 of
+// L = 8 729, 723, 737, 755; 12 of L = 10 1530, 1480, 1483, 1502; 12 runs of 2D L = 16 618, 649,
+// 633, 635; L = 32 2356, 2406, 2359, 2380; a serving batch 1772, 1802, 1829, 1900.
+template <int DIM, int L, int RSP>
+__host__ __device__ constexpr int resident() {
+    constexpr int n = (DIM == 3 ? 640 : 512) / Team<DIM, L, RSP>::TT;
+    return n < 1 ? 1 : n;
+}
 // Each team claims a chunk at a time and stages its run's round keys and
 // coupling patterns.
 template <int DIM, int L, bool PMJ, int RSP>
-__global__ void __launch_bounds__(Team<DIM, L, RSP>::TT) k_sweep_team_batched(BatchSweepArgs a) {
+__global__ void __launch_bounds__(Team<DIM, L, RSP>::TT, resident<DIM, L, RSP>())
+    k_sweep_team_batched(BatchSweepArgs a) {
     extern __shared__ uint4 smem[];
     __shared__ uint32_t s_chunk;
     constexpr int SQ = s_quads<DIM, L>();
