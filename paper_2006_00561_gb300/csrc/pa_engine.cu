@@ -309,41 +309,44 @@ void thresholds_into(double beta, uint32_t* t4) {
     t4[3] = full;
 }
 
-// Moves step i of the schedule to inverse temperature b, with temperature step
-// b - beta[i-1]: the thresholds, beta and dbeta of step i are replaced, and its
-// weight table goes to dynamic slot i & 1 unless the fixed schedule already
-// has this exact step.  Host copies first, then stream-ordered uploads.
+// Host copies of step i at inverse temperature b, with temperature step b -
+// beta[i-1]: its thresholds, beta, dbeta and the weight table it takes, dynamic
+// slot i & 1 unless the fixed schedule already has this exact step.  A new
+// dynamic table is uploaded.
 int set_step(pa_run* r, uint32_t i, double b, cudaStream_t s) {
     RunDev& d = r->d;
     r->beta[i] = b;
     thresholds_into(b, &r->thr[(size_t)i * 4]);
-    if (i >= 1) {
-        r->dbeta[i] = b - r->beta[i - 1];
-        if (r->dbeta[i] == r->dbeta_fixed[i]) {
-            r->dsel[i] = r->dsel_fixed[i];
-        } else {
-            std::vector<double>& t = r->dyn_table[i & 1];
-            t.resize((size_t)d.bins);
-            for (int64_t j = 0; j < d.bins; ++j) t[j] = weight_of(r->dbeta[i], j);
-            r->dsel[i] = r->ndist + (i & 1);
-            CK(cudaMemcpyAsync((void*)(d.dtab + (size_t)r->dsel[i] * d.bins), t.data(),
-                               (size_t)d.bins * 8, cudaMemcpyHostToDevice, s));
-        }
-        CK(cudaMemcpyAsync((void*)(d.dbeta + i), &r->dbeta[i], 8, cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync((void*)(d.dsel + i), &r->dsel[i], 4, cudaMemcpyHostToDevice, s));
+    if (i < 1) return PA_OK;
+    r->dbeta[i] = b - r->beta[i - 1];
+    if (r->dbeta[i] == r->dbeta_fixed[i]) {
+        r->dsel[i] = r->dsel_fixed[i];
+        return PA_OK;
     }
-    CK(cudaMemcpyAsync((void*)(d.beta + i), &r->beta[i], 8, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync((void*)(d.thr + (size_t)i * 4), &r->thr[(size_t)i * 4], 16,
+    std::vector<double>& t = r->dyn_table[i & 1];
+    t.resize((size_t)d.bins);
+    for (int64_t j = 0; j < d.bins; ++j) t[j] = weight_of(r->dbeta[i], j);
+    r->dsel[i] = r->ndist + (i & 1);
+    CK(cudaMemcpyAsync((void*)(d.dtab + (size_t)r->dsel[i] * d.bins), t.data(), (size_t)d.bins * 8,
                        cudaMemcpyHostToDevice, s));
     return PA_OK;
 }
 
-// Step i at beta_i; step i + 1 keeps its fixed beta, with its temperature step
-// taken from beta_i.
+// Moves step i of the schedule to inverse temperature b; step i + 1 keeps its
+// fixed beta, with its temperature step taken from b.  Host copies first, then
+// stream-ordered uploads, one per array for both steps.
 int move_step(pa_run* r, uint32_t i, double b, cudaStream_t s) {
+    RunDev& d = r->d;
     int rc = set_step(r, i, b, s);
-    if (rc == PA_OK && i + 1 <= (uint32_t)r->cfg.K) rc = set_step(r, i + 1, r->beta_fixed[i + 1], s);
-    return rc;
+    const size_t n = i + 1 <= (uint32_t)r->cfg.K ? 2 : 1;
+    if (rc == PA_OK && n == 2) rc = set_step(r, i + 1, r->beta_fixed[i + 1], s);
+    if (rc) return rc;
+    CK(cudaMemcpyAsync((void*)(d.dbeta + i), &r->dbeta[i], n * 8, cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync((void*)(d.dsel + i), &r->dsel[i], n * 4, cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync((void*)(d.beta + i), &r->beta[i], n * 8, cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync((void*)(d.thr + (size_t)i * 4), &r->thr[(size_t)i * 4], n * 16,
+                       cudaMemcpyHostToDevice, s));
+    return PA_OK;
 }
 
 int enqueue_step(pa_run* r, cudaStream_t s) {
@@ -1020,40 +1023,46 @@ int pa_restore(pa_run* r, const void* src, size_t bytes) {
     return PA_OK;
 }
 
-// Histogram overlap of the population with its reweighting to beta + dbeta:
-// sum_k min(H_k / R, H_k w_k / sum_j H_j w_j), sums over k ascending.
-static double overlap_of(const std::vector<uint32_t>& H, int64_t R, double dbeta) {
-    const bool heating = dbeta < 0.0;
-    const int64_t bins = (int64_t)H.size();
-    int64_t kref = -1;
-    if (heating) {
-        for (int64_t k = bins - 1; k >= 0; --k)
-            if (H[k]) {
-                kref = k;
-                break;
-            }
-    } else {
-        for (int64_t k = 0; k < bins; ++k)
-            if (H[k]) {
-                kref = k;
-                break;
-            }
+// The occupied levels of a histogram, ascending, for steps of one sign: how far
+// each lies from the reference level (lowest occupied when cooling, highest when
+// heating), H_k and H_k / R.
+struct Occupied {
+    std::vector<int64_t> j;
+    std::vector<double> H, p, hw;
+};
+
+static void occupied_levels(const std::vector<uint32_t>& hist, int64_t R, bool heating, Occupied& o) {
+    int64_t first = -1, last = -1;
+    for (int64_t k = 0; k < (int64_t)hist.size(); ++k) {
+        if (!hist[k]) continue;
+        if (first < 0) first = k;
+        last = k;
+        o.j.push_back(k);
+        o.H.push_back((double)hist[k]);
+        o.p.push_back((double)hist[k] / (double)R);
     }
-    if (kref < 0 || R < 1) return 0.0;
+    for (int64_t& k : o.j) k = heating ? last - k : k - first;
+    o.hw.resize(o.j.size());
+}
+
+// Whether the overlap of the population with its reweighting to beta + dbeta,
+// sum_k min(H_k / R, H_k w_k / sum_j H_j w_j) with sums over k ascending, is at
+// least `target`.  The terms are not negative, so the sum can only grow.
+static bool overlaps(Occupied& o, double dbeta, double target) {
+    const size_t n = o.j.size();
     double sw = 0.0;
-    for (int64_t k = 0; k < bins; ++k) {
-        const int64_t j = heating ? kref - k : k - kref;
-        if (j >= 0 && H[k]) sw = sw + (double)H[k] * weight_of(dbeta, j);
+    for (size_t q = 0; q < n; ++q) {
+        o.hw[q] = o.H[q] * weight_of(dbeta, o.j[q]);
+        sw = sw + o.hw[q];
     }
     double a = 0.0;
-    for (int64_t k = 0; k < bins; ++k) {
-        const int64_t j = heating ? kref - k : k - kref;
-        if (j < 0 || !H[k]) continue;
-        const double p = (double)H[k] / (double)R;
-        const double q = ((double)H[k] * weight_of(dbeta, j)) / sw;
-        a = a + (p < q ? p : q);
+    if (a >= target) return true;
+    for (size_t q = 0; q < n; ++q) {
+        const double w = o.hw[q] / sw;
+        a = a + (o.p[q] < w ? o.p[q] : w);
+        if (a >= target) return true;
     }
-    return a;
+    return false;
 }
 
 int pa_adaptive_beta(pa_run* r, double target, double beta_end, double* beta_next) {
@@ -1067,7 +1076,9 @@ int pa_adaptive_beta(pa_run* r, double target, double beta_end, double* beta_nex
     CK(cudaMemcpy(H.data(), r->d.hist, H.size() * 4, cudaMemcpyDeviceToHost));
     const double beta = r->beta[st.step];
     const double span = beta_end - beta;
-    if (span == 0.0 || overlap_of(H, st.R, span) >= target) {
+    Occupied o;
+    occupied_levels(H, st.R, span < 0.0, o);
+    if (span == 0.0 || overlaps(o, span, target)) {
         *beta_next = span == 0.0 ? beta : beta_end;
         return PA_OK;
     }
@@ -1075,7 +1086,7 @@ int pa_adaptive_beta(pa_run* r, double target, double beta_end, double* beta_nex
     const double sgn = span < 0.0 ? -1.0 : 1.0;
     for (int it = 0; it < 60; ++it) {
         const double mid = lo + (hi - lo) * 0.5;
-        if (overlap_of(H, st.R, sgn * mid) >= target) lo = mid;
+        if (overlaps(o, sgn * mid, target)) lo = mid;
         else hi = mid;
     }
     *beta_next = beta + sgn * lo;
