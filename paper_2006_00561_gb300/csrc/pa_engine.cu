@@ -482,6 +482,9 @@ int pa_init(const pa_config* cfg, void* ws, size_t bytes, void* stream, pa_run**
     d.R0 = (uint32_t)cfg->R0;
     d.tiles = (uint32_t)l.tiles;
     d.slice_lg = pa::resample_slices((uint64_t)l.stride, (uint64_t)l.cap * l.stride, 1u << 14);
+    double largest = 0.0;
+    for (double x : dbeta) largest = std::fabs(x) > largest ? std::fabs(x) : largest;
+    d.spread = pa::many_copies(largest, (double)(cfg->dim * l.N)) ? 1u : 0u;
     d.mn_cum = l.mn_cum ? (unsigned long long*)(base + l.mn_cum) : nullptr;
     d.mn_tiles = l.mn_tiles ? (unsigned long long*)(base + l.mn_tiles) : nullptr;
     r->hist_bytes = 16 + (size_t)l.bins * 4;
@@ -989,6 +992,7 @@ int pa_restore(pa_run* r, const void* src, size_t bytes) {
     st.epoch = now.epoch;
     st.tile_counter = 0;
     st.tau_done = 0;
+    st.over_n = 0;
     st.active = 0;
     st.status = 0;
     r->init_state = st;
@@ -1454,9 +1458,11 @@ int batch_init(pa_run* const* runs, int32_t nruns, const int32_t* steps_left, vo
     b->bd.max_bins = 1;
     for (const auto& h : h_runs)
         if (h.bins > b->bd.max_bins) b->bd.max_bins = h.bins;
+    b->bd.any_spread = 0;
     b->bd.any_poisson = 0;
     b->bd.any_multinomial = 0;
     for (const auto& h : h_runs) {
+        if (h.spread) b->bd.any_spread = 1;
         if (h.resample == PA_RESAMPLE_POISSON) b->bd.any_poisson = 1;
         if (h.resample == PA_RESAMPLE_MULTINOMIAL) {
             b->bd.any_multinomial = 1;

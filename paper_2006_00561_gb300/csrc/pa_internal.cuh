@@ -47,7 +47,8 @@ struct DevState {
     unsigned long long sweeps_done;
     unsigned long long tau_done;  // CTAs of the running multi-CTA reweight that are done
     unsigned long long sources;   // replicas with a copy count > 0, summed over all resamples
-    unsigned long long pad[1];
+    uint32_t over_n;              // copies left to k_spread: entries of RunDev::srcmap2
+    uint32_t pad;
 };
 static_assert(sizeof(DevState) <= 256, "DevState must fit its slot");
 
@@ -65,7 +66,8 @@ struct RunDev {
     uint32_t* counts;           // copy counts of the last resample
     uint32_t* offsets;          // exclusive scan of the counts
     uint32_t* srcmap;           // [cap] source replica of every slot the last resample filled
-    uint32_t* srcmap2;          // [cap] the same after a redistribution permuted the slots
+    uint32_t* srcmap2;          // [cap] the same after a redistribution permuted the slots;
+                                // in a whole resample the list of k_spread
     unsigned long long* accum;  // [2] = sum |M|, sum M^2 of the running measurement
     uint32_t* hist;             // [bins] energy histogram of the running measurement
     uint32_t* tab_n;            // [bins] floor(tau_k)
@@ -107,6 +109,7 @@ struct RunDev {
     // the resample clears the histogram and the magnetisation sums for the sweep
     // that follows it (whole steps; a lone resample leaves them)
     uint32_t clear_hist;
+    uint32_t spread;  // replicas may get many copies: k_spread shares them out (many_copies)
 };
 
 // A batch of runs stepped together (pa_batch_* in include/pa.h).  Arrays in
@@ -118,6 +121,7 @@ struct BatchDev {
     int64_t max_bins;            // energy levels of the run with the most
     const uint32_t* tile_base;   // [nruns + 1] prefix sums of each run's slices of tiles
     uint32_t total_tiles;        // slices of all tiles
+    uint32_t any_spread;         // some run's RunDev::spread is set
     uint32_t any_poisson;        // some run resamples by the Poisson rule
     uint32_t any_multinomial;    // some run resamples by multinomial draws
     uint32_t* counters;          // [0]: resample tiles, [1 + c]: sweep chunks of class c
@@ -349,6 +353,18 @@ inline uint32_t resample_slices(uint64_t stride, uint64_t total, uint64_t least)
     uint32_t lg = 0;
     while (((uint32_t)RS_TILE >> (lg + 1)) >= 32 && ((uint64_t)RS_TILE >> lg) * stride > target) ++lg;
     return lg;
+}
+
+// A replica's copies are written by one CTA as long as they are few.  With beta
+// steps of twice the inverse of the energy's standard deviation (sqrt(dim N) at
+// beta = 0) and more a few replicas get hundreds of copies and then most of the
+// population: the CTAs that hold them leave all copies beyond the first
+// SPREAD_FROM, in entries of SPREAD_COPIES, to k_spread, which shares the entries
+// out to all CTAs.  Such runs have kernels of their own: the code for it costs
+// every resample about a microsecond.
+constexpr uint32_t SPREAD_FROM = 16, SPREAD_COPIES = 64;
+inline bool many_copies(double largest_dbeta, double bonds) {
+    return largest_dbeta * largest_dbeta * bonds > 4.0;
 }
 
 }  // namespace pa

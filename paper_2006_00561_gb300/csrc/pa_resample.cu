@@ -236,6 +236,7 @@ __device__ __forceinline__ bool tau_run(const RunDev& d, uint32_t blk, uint32_t 
         st->R_prev = R;
         st->epoch = epoch + 1;
         st->tile_counter = 0;
+        st->over_n = 0;
         st->src = cur;
         st->cur = cur ^ 1u;
         st->active = 1;
@@ -370,6 +371,57 @@ __global__ void __launch_bounds__(RS_THREADS) k_poisson_counts_batched(BatchDev 
     if (base < R) poisson_counts(s_d, base + threadIdx.x, RS_THREADS, min(R, base + width));
 }
 
+// Entries of k_spread: {source replica, first slot, copies}, at most
+// SPREAD_COPIES copies each.  Copies beyond the capacity are dropped here as they
+// are everywhere; what is left fits the list (one entry per 17 copies at least).
+__device__ __forceinline__ void leave_copies(const RunDev& d, uint32_t src, uint32_t dst, uint32_t n) {
+    if (dst >= d.cap) return;
+    n = min(n, d.cap - dst);
+    const uint32_t m = (n + SPREAD_COPIES - 1) / SPREAD_COPIES, room = d.cap_alloc / 3u;
+    const uint32_t e0 = atomicAdd(&d.st->over_n, m);
+    for (uint32_t e = 0; e < m && e0 + e < room; ++e) {
+        uint32_t* at = d.srcmap2 + 3 * (size_t)(e0 + e);
+        at[0] = src;
+        at[1] = dst + e * SPREAD_COPIES;
+        at[2] = min(SPREAD_COPIES, n - e * SPREAD_COPIES);
+    }
+}
+
+// The copies that the resample's CTAs have left: blk of nblk CTAs takes entries
+// blk, blk + nblk, ...  Measured on GB300: the batched resample of a serving batch
+// (163 000 replicas, beta steps up to seven standard deviations of the energy at L =
+// 128) takes 35 us with it and 115 without, when one CTA wrote thousands of copies of a
+// replica.
+__device__ __forceinline__ void spread_run(const RunDev& d, uint32_t blk, uint32_t nblk) {
+    const DevState* st = d.st;
+    const uint32_t n = min(st->over_n, d.cap_alloc / 3u), src = st->src;
+    const uint32_t CH = d.stride >> 4;
+    for (uint32_t e = blk; e < n; e += nblk) {
+        const uint32_t* at = d.srcmap2 + 3 * (size_t)e;
+        const uint32_t rep = at[0], dst = at[1], copies = at[2];
+        const uint4* __restrict__ from = reinterpret_cast<const uint4*>(d.spins[src]) + (size_t)rep * CH;
+        uint4* __restrict__ to = reinterpret_cast<uint4*>(d.spins[src ^ 1u]) + (size_t)dst * CH;
+        for (uint32_t it = threadIdx.x; it < copies * CH; it += 256) __stcs(to + it, __ldg(from + it % CH));
+        const uint32_t level = d.ebin[src][rep];
+        const int32_t mag = d.mag[src][rep];
+        for (uint32_t k = threadIdx.x; k < copies; k += 256) {
+            d.ebin[src ^ 1u][dst + k] = level;
+            d.mag[src ^ 1u][dst + k] = mag;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(256) k_spread(__grid_constant__ const RunDev d) {
+    chain_wait();
+    if (d.st->active) spread_run(d, blockIdx.x, gridDim.x);
+}
+
+// Batched: column r of the grid serves run r.
+__global__ void __launch_bounds__(256) k_spread_batched(BatchDev b) {
+    const RunDev& d = b.runs[blockIdx.x];
+    if (d.st->active && d.st->over_n) spread_run(d, blockIdx.y, gridDim.y);
+}
+
 // RULE 0 compiles the nearest-integer rule alone (the register budget of the
 // HBM-bound default path); 2 takes the counts that the Poisson or multinomial
 // draws have left in d.counts; 3 chooses between the two per run (batches).
@@ -379,7 +431,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_poisson_counts_batched(BatchDev 
 // source replica (srcmap) with the copied energy level and magnetisation, and
 // k_gather copies the spins afterwards over the whole new population (the
 // plain form).
-template <int RULE, bool SPLIT = false>
+template <int RULE, bool SPLIT, bool SPREAD>
 __device__ __forceinline__ void resample_tile(const RunDev& d, uint32_t tile, uint32_t slice,
                                               ResampleSmem& sm) {
     DevState* st = d.st;
@@ -496,9 +548,14 @@ __device__ __forceinline__ void resample_tile(const RunDev& d, uint32_t tile, ui
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            if (r[j0 + j]) {  // 0 beyond R
+            uint32_t c = r[j0 + j];
+            if (c) {  // 0 beyond R
+                if (SPREAD && c > SPREAD_FROM) {
+                    leave_copies(d, i0 + j, oo[j] + SPREAD_FROM, c - SPREAD_FROM);
+                    c = SPREAD_FROM;
+                }
                 sm.surv[p] = li0 + j;
-                sm.r[p] = r[j0 + j];
+                sm.r[p] = c;
                 sm.o[p++] = oo[j];
             }
         }
@@ -592,7 +649,7 @@ __device__ __forceinline__ void resample_tile(const RunDev& d, uint32_t tile, ui
 #ifndef PA_RS_MINB
 #define PA_RS_MINB 4
 #endif
-template <int RULE, bool SPLIT>
+template <int RULE, bool SPLIT, bool SPREAD>
 __global__ void __launch_bounds__(RS_THREADS, PA_RS_MINB) k_resample(__grid_constant__ const RunDev d) {
     __shared__ ResampleSmem sm;
     chain_wait();
@@ -612,7 +669,7 @@ __global__ void __launch_bounds__(RS_THREADS, PA_RS_MINB) k_resample(__grid_cons
     for (;;) {
         const uint32_t id = sm.tile, tile = id >> d.slice_lg;
         if (tile >= (R + (uint32_t)RS_TILE - 1) / (uint32_t)RS_TILE) break;
-        resample_tile<RULE, SPLIT>(d, tile, id & ((1u << d.slice_lg) - 1u), sm);
+        resample_tile<RULE, SPLIT, SPREAD>(d, tile, id & ((1u << d.slice_lg) - 1u), sm);
         if (single) break;
         __syncthreads();  // sm is reused by the next tile
         if (threadIdx.x == 0) sm.tile = atomicAdd(&d.st->tile_counter, 1u);
@@ -747,7 +804,7 @@ __global__ void __launch_bounds__(256) k_remap(RunDev d, const __grid_constant__
 // Batched: global tile ids are claimed in increasing order; run r owns ids
 // tile_base[r] .. tile_base[r+1]-1, so within a run tiles are claimed in order
 // and the lookback only ever waits on tiles already running.
-template <int RULE>
+template <int RULE, bool SPREAD>
 __global__ void __launch_bounds__(RS_THREADS, PA_RS_MINB) k_resample_batched(BatchDev b) {
     __shared__ ResampleSmem sm;
     __shared__ uint32_t s_run;
@@ -784,7 +841,7 @@ __global__ void __launch_bounds__(RS_THREADS, PA_RS_MINB) k_resample_batched(Bat
         const RunDev& d = b.runs[s_run];
 #endif
         if (d.st->active)
-            resample_tile<RULE>(d, sm.tile >> d.slice_lg, sm.tile & ((1u << d.slice_lg) - 1u), sm);
+            resample_tile<RULE, false, SPREAD>(d, sm.tile >> d.slice_lg, sm.tile & ((1u << d.slice_lg) - 1u), sm);
         __syncthreads();
     }
 }
@@ -892,7 +949,7 @@ cudaError_t launch_tau(const RunDev& d, cudaStream_t s) {
 // One wave of resident CTAs (capped by the number of tiles), looked up once
 // per device and kernel.
 static int resample_wave(const void* fn, int which, uint32_t tiles) {
-    static int cache[64][10];
+    static int cache[64][12];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
     int wave = cache[dev][which];
@@ -958,9 +1015,14 @@ static cudaError_t launch_counts_scan(const RunDev& d, cudaStream_t s) {
         if (e != cudaSuccess) return e;
     }
     const bool drawn = d.resample != PA_RESAMPLE_NEAREST;
-    const void* fn = drawn ? (const void*)k_resample<2, SPLIT> : (const void*)k_resample<0, SPLIT>;
-    // cache slots: 0 and 4 the one-kernel forms, 7 and 9 the split forms
-    const int grid = resample_wave(fn, SPLIT ? (drawn ? 9 : 7) : (drawn ? 4 : 0),
+    const bool spread = !SPLIT && d.spread;
+    const void* fn = drawn ? (spread ? (const void*)k_resample<2, SPLIT, !SPLIT>
+                                     : (const void*)k_resample<2, SPLIT, false>)
+                           : (spread ? (const void*)k_resample<0, SPLIT, !SPLIT>
+                                     : (const void*)k_resample<0, SPLIT, false>);
+    // cache slots: 0 and 4 the one-kernel forms (2 and 3 with k_spread), 7 and 9
+    // the split forms
+    const int grid = resample_wave(fn, SPLIT ? (drawn ? 9 : 7) : spread ? (drawn ? 3 : 2) : (drawn ? 4 : 0),
                                    d.tiles << d.slice_lg);
     if (grid <= 0) return cudaErrorInvalidValue;
     return launch_chained(fn, dim3(grid), dim3(RS_THREADS), 0, s, args);
@@ -968,6 +1030,11 @@ static cudaError_t launch_counts_scan(const RunDev& d, cudaStream_t s) {
 
 cudaError_t launch_resample(const RunDev& d, cudaStream_t s) {
     cudaError_t e = launch_counts_scan<RS_SPLIT>(d, s);
+    if (e == cudaSuccess && !RS_SPLIT && d.spread) {
+        RunDev dd = d;
+        void* args[] = {&dd};
+        e = launch_chained((const void*)k_spread, dim3(RS_CTAS), dim3(256), 0, s, args);
+    }
     if (e != cudaSuccess || !RS_SPLIT) return e;
     const int g = gather_grid();
     if (g <= 0) return cudaErrorInvalidValue;
@@ -1177,15 +1244,18 @@ cudaError_t launch_resample_batched(const BatchDev& b, cudaStream_t s) {
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    if (b.any_poisson || b.any_multinomial) {
-        const int grid = resample_wave((const void*)k_resample_batched<3>, 6, b.total_tiles);
-        if (grid <= 0) return cudaErrorInvalidValue;
-        k_resample_batched<3><<<grid, RS_THREADS, 0, s>>>(b);
-    } else {
-        const int grid = resample_wave((const void*)k_resample_batched<0>, 1, b.total_tiles);
-        if (grid <= 0) return cudaErrorInvalidValue;
-        k_resample_batched<0><<<grid, RS_THREADS, 0, s>>>(b);
-    }
+    const bool drawn = b.any_poisson || b.any_multinomial;
+    const void* fn = drawn ? (b.any_spread ? (const void*)k_resample_batched<3, true>
+                                           : (const void*)k_resample_batched<3, false>)
+                           : (b.any_spread ? (const void*)k_resample_batched<0, true>
+                                           : (const void*)k_resample_batched<0, false>);
+    const int grid = resample_wave(fn, b.any_spread ? (drawn ? 11 : 10) : (drawn ? 6 : 1), b.total_tiles);
+    if (grid <= 0) return cudaErrorInvalidValue;
+    BatchDev bb = b;
+    void* args[] = {&bb};
+    const cudaError_t e = cudaLaunchKernel(fn, dim3(grid), dim3(RS_THREADS), args, 0, s);
+    if (e != cudaSuccess) return e;
+    if (b.any_spread) k_spread_batched<<<dim3(b.nruns, 32), 256, 0, s>>>(b);
     return cudaGetLastError();
 }
 

@@ -96,3 +96,31 @@ def test_allocation_free_scan_at_any_alignment(P, R, shift):
     assert int(total.cpu().numpy().view(np.uint32)[0]) == int(want.astype(np.int64).sum())
     for a in (counts, offsets):  # nothing outside the caller's range is written
         assert (a[:shift] == 0xffffffff).all() and (a[shift + R:] == 0xffffffff).all()
+
+
+SKEWED = [dict(dim=2, L=32, layout=1, R0=3000, K=4, beta_max=2.0), dict(dim=2, L=16, layout=0, R0=5000, K=6),
+          dict(dim=3, L=6, layout=1, model=1, coupling_seed=9, R0=2100, K=3, beta_max=3.0),
+          dict(dim=2, L=64, layout=1, R0=700, K=40), dict(dim=2, L=4, layout=1, R0=9000, K=2, beta_max=3.0)]
+
+
+@pytest.mark.parametrize("rule", [0, 1, 2])
+@pytest.mark.parametrize("spec", SKEWED, ids=lambda s: f"{s['dim']}d L={s['L']}")
+def test_beta_steps_that_leave_few_survivors(P, spec, rule):
+    """Replicas with tens to thousands of copies, shared out to all CTAs."""
+    run_lockstep(P, steps=2, theta=1, seed=31, resample=rule, **spec)
+
+
+def test_batch_with_few_survivors(P):
+    runs, oracles = [], []
+    for i, s in enumerate(SKEWED + [dict(dim=2, L=16, layout=1, R0=300, K=50)]):
+        ocfg, gcfg = configs(P, theta=1, seed=50 + i, resample=i % 3, **s)
+        oracles.append(O.Run(ocfg))
+        runs.append(P.Run(gcfg))
+    batch = P.Batch(runs)
+    for i in (1, 2):
+        batch.step()
+        assert batch.sync() == 0
+        for r, o in zip(runs, oracles):
+            assert o.step() == 0
+            compare_state(P, r, o, i)
+    batch.close()
