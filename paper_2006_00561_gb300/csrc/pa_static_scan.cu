@@ -37,8 +37,9 @@ static __device__ __align__(256) StaticScanScratch g_scan_scratch;
 // lookback saves re-reading the counts, but its prefix moves from tile to
 // tile in L2 round trips: 3 000 017 replicas (1465 tiles) took 64.4 us on GB300
 // with one descriptor at a time, 51.2 us with 32, 42.6 us with 256; the two passes
-// take 18.0 us a call (2.0 TB/s over the caller's arrays: launches and the two
-// dependent L2 round trips of each pass bound it).
+// take 12.4 us a call (2.9 TB/s over the caller's arrays), 16.4 as single launches
+// instead of a chain; up to 10^6 replicas a call is 6.1 to 6.6 us (8.2 to 12.3), its
+// launches and each pass's two dependent L2 round trips.
 //
 // VEC: the caller's three arrays are 16-byte aligned, so a thread's eight
 // replicas move as 16-byte words.
@@ -49,6 +50,7 @@ __global__ void __launch_bounds__(SS_THREADS)
                     uint32_t bins, uint32_t step, uint32_t ctr3, uint32_t k0, uint32_t k1,
                     uint32_t* __restrict__ counts) {
     __shared__ uint32_t s_warp[SS_THREADS / 32];
+    chain_wait();
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const uint32_t base = blockIdx.x * SS_TILE;
     uint32_t sum = 0;
@@ -102,6 +104,7 @@ __global__ void __launch_bounds__(SS_THREADS)
     k_static_offsets(const StaticScanScratch* __restrict__ s, const uint32_t* __restrict__ counts,
                      uint32_t R, uint32_t* __restrict__ offsets, uint32_t* __restrict__ total) {
     __shared__ uint32_t s_warp[SS_THREADS / 32], s_before[SS_THREADS / 32];
+    chain_wait();
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const uint32_t tile = blockIdx.x, base = tile * SS_TILE;
     uint32_t r[SS_ITEMS];
@@ -264,13 +267,14 @@ extern "C" int pa_copy_counts_scan_noalloc(const uint32_t* d_ebin, int64_t R,
     const uint32_t tiles = (uint32_t)((R + pa::SS_TILE - 1) / pa::SS_TILE);
     const uint32_t ctr3 = (pa::TAG_RESAMPLE << 28) | (uint32_t)instance_id;
     const bool vec = (((uintptr_t)d_ebin | (uintptr_t)d_counts | (uintptr_t)d_offsets) & 15u) == 0;
-    auto* count = vec ? pa::k_static_counts<true> : pa::k_static_counts<false>;
-    auto* scan = vec ? pa::k_static_offsets<true> : pa::k_static_offsets<false>;
-    count<<<tiles, pa::SS_THREADS, 0, st>>>(s, d_ebin, (uint32_t)R, d_tab_n, d_tab_F, (uint32_t)bins,
-                                            (uint32_t)step, ctr3, (uint32_t)seed,
-                                            (uint32_t)(seed >> 32), d_counts);
-    if (cudaGetLastError() != cudaSuccess) return PA_ERR_CUDA;
-    scan<<<tiles, pa::SS_THREADS, 0, st>>>(s, d_counts, (uint32_t)R, d_offsets, d_total);
-    if (cudaGetLastError() != cudaSuccess) return PA_ERR_CUDA;
+    const void* count = vec ? (const void*)pa::k_static_counts<true> : (const void*)pa::k_static_counts<false>;
+    const void* scan = vec ? (const void*)pa::k_static_offsets<true> : (const void*)pa::k_static_offsets<false>;
+    uint32_t r = (uint32_t)R, nb = (uint32_t)bins, st32 = (uint32_t)step, c3 = ctr3;
+    uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+    void* cargs[] = {&s, &d_ebin, &r, &d_tab_n, &d_tab_F, &nb, &st32, &c3, &k0, &k1, &d_counts};
+    void* sargs[] = {&s, &d_counts, &r, &d_offsets, &d_total};
+    if (pa::launch_chained(count, dim3(tiles), dim3(pa::SS_THREADS), 0, st, cargs) != cudaSuccess ||
+        pa::launch_chained(scan, dim3(tiles), dim3(pa::SS_THREADS), 0, st, sargs) != cudaSuccess)
+        return PA_ERR_CUDA;
     return PA_OK;
 }

@@ -57,7 +57,8 @@ constexpr int WARPS64 = PA_L64_WARPS;
 // than all warps of a few.  us per launch on GB300 (theta = 10), 12 warps with a
 // block's replicas together -> apart at 8, 12, 16 warps: 256 replicas 50 -> 26, 25,
 // 25; 20480 521 -> 502, 494, 489 (theta = 1: 61 -> 64, 61, 58); 2^20 24596 -> 25201, 24469,
-// 24371; +-J 2^20 25121 -> 25648, 24993, 25092.
+// 24371; +-J 2^20 25121 -> 25648, 24993, 25092.  20 and 24 warps (96 and 80 registers) run
+// 2^20 replicas in 24553 and 24599, 18 in 27270 (the schedulers' shares differ).
 constexpr int WARPS64_FERRO = 16, WARPS64_PMJ = 12;
 
 __device__ __forceinline__ uint64_t shfl64(uint64_t v, int src) {
