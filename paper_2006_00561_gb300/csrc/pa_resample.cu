@@ -1061,9 +1061,8 @@ cudaError_t launch_remap_gather(const RunDev& d, const SegList& segs, cudaStream
 // ---------------------------------------------------------------------------
 // Multinomial resampling: the copy counts of all replicas come from R0
 // independent draws.  Replica i weighs t_i = n_k 2^32 + F_k (k = its level);
-// C_i = t_0 + ... + t_i are exact 64-bit integers, built by a three-pass scan
-// over tiles of RS_TILE replicas (tile sums, one-CTA scan of the tile sums,
-// per-tile prefix).  Draw j: v = words 2(j & 1) (low) and 2(j & 1) + 1 (high)
+// C_i = t_0 + ... + t_i are exact 64-bit integers, built by a two-pass scan over
+// tiles of RS_TILE replicas (tile sums, then the prefix of each tile).  Draw j: v = words 2(j & 1) (low) and 2(j & 1) + 1 (high)
 // of Philox block (j >> 1, step, 0, MULTINOMIAL|id), x = floor(v C_{R-1} /
 // 2^64), one copy (atomic add) to the first replica with C_i > x.
 // ---------------------------------------------------------------------------
@@ -1102,37 +1101,9 @@ __global__ void __launch_bounds__(RS_THREADS) k_mn_tile_sums(__grid_constant__ c
     }
 }
 
-// Exclusive scan of the tile sums in place; mn_tiles[ntiles] = the total.
-__global__ void __launch_bounds__(1024) k_mn_scan(__grid_constant__ const RunDev d) {
-    __shared__ unsigned long long s[1024];
-    chain_wait();
-    const DevState* st = d.st;
-    if (!st->active) return;
-    const uint32_t R = st->R_prev;
-    const uint32_t ntiles = (R + RS_TILE - 1) / RS_TILE;
-    const uint32_t t = threadIdx.x;
-    const uint32_t per = (ntiles + 1023) / 1024;
-    const uint32_t lo = t * per, hi = min(ntiles, lo + per);
-    unsigned long long part = 0;
-    for (uint32_t k = lo; k < hi; ++k) part += d.mn_tiles[k];
-    s[t] = part;
-    __syncthreads();
-    for (uint32_t o = 1; o < 1024; o <<= 1) {  // inclusive Hillis-Steele scan
-        const unsigned long long v = t >= o ? s[t - o] : 0ull;
-        __syncthreads();
-        s[t] += v;
-        __syncthreads();
-    }
-    unsigned long long run = s[t] - part;
-    for (uint32_t k = lo; k < hi; ++k) {
-        const unsigned long long v = d.mn_tiles[k];
-        d.mn_tiles[k] = run;
-        run += v;
-    }
-    if (t == 1023) d.mn_tiles[ntiles] = s[1023];
-}
-
-// C_i per replica (inclusive), and the copy counts cleared for the draws.
+// C_i per replica (inclusive), and the copy counts cleared for the draws.  A CTA
+// adds up the sums of the tiles before its own itself (a few independent loads a
+// thread); mn_tiles[ntiles] = the total.
 __global__ void __launch_bounds__(RS_THREADS) k_mn_cum(__grid_constant__ const RunDev d) {
     __shared__ unsigned long long sw[RS_THREADS / 32];
     chain_wait();
@@ -1156,9 +1127,16 @@ __global__ void __launch_bounds__(RS_THREADS) k_mn_cum(__grid_constant__ const R
             const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += y;
         }
+        unsigned long long ahead = 0;
+        for (uint32_t k = threadIdx.x; k < tile; k += RS_THREADS) ahead += d.mn_tiles[k];
+        unsigned long long before = block_sum_u64(ahead, sw);
         if (lane == 31) sw[wid] = incl;
         __syncthreads();
-        unsigned long long before = d.mn_tiles[tile];
+        if (tile == ntiles - 1 && threadIdx.x == 0) {
+            unsigned long long all = before;
+            for (int k = 0; k < RS_THREADS / 32; ++k) all += sw[k];
+            d.mn_tiles[ntiles] = all;
+        }
         for (int k = 0; k < wid; ++k) before += sw[k];
         unsigned long long run = before + incl - part;
 #pragma unroll
@@ -1217,7 +1195,6 @@ cudaError_t launch_multinomial(const RunDev& d, cudaStream_t s) {
         const void* fn;
         int grid, threads;
     } pass[] = {{(const void*)k_mn_tile_sums, wave, RS_THREADS},
-                {(const void*)k_mn_scan, 1, 1024},
                 {(const void*)k_mn_cum, wave, RS_THREADS},
                 {(const void*)k_mn_draw, g, 256}};
     for (const auto& p : pass) {
