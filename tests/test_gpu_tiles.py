@@ -124,3 +124,9 @@ def test_batch_with_few_survivors(P):
             assert o.step() == 0
             compare_state(P, r, o, i)
     batch.close()
+
+
+@pytest.mark.parametrize("R0", [2047, 2048, 6145, 400_003])
+def test_multinomial_draws_over_several_tiles(P, R0):
+    run_lockstep(P, steps=2, dim=2, L=4, layout=1, R0=R0, K=8, theta=1, beta_max=1.0, seed=R0,
+                 resample=2)
