@@ -59,9 +59,9 @@ constexpr size_t ALIGN = 256;
 
 // Steps in the CUDA graph of pa_run_steps, and the steps of a call from which
 // one is built.  Chained launches run a step as fast as the graph does (31.8
-// against 31.7 us for 1000 replicas at L = 16 on GB300, 39 us with a graph of one
-// step), and the graph's construction and first launch cost 100 us; a long call
-// takes it to leave the host free (1.5 us a step instead of 7.5).
+// against 31.7 us for 1000 replicas at L = 16 on GB300 when this was measured, 39 us
+// with a graph of one step), and the graph's construction and first launch cost
+// 100 us; a long call takes it to leave the host free (1.5 us a step instead of 7.5).
 constexpr int32_t GRAPH_STEPS = 8, GRAPH_FROM = 256;
 
 size_t align_up(size_t v) { return (v + ALIGN - 1) / ALIGN * ALIGN; }
@@ -353,6 +353,21 @@ int enqueue_step(pa_run* r, cudaStream_t s) {
     int rc = enqueue_resample(r, s, true);
     if (rc) return rc;
     return enqueue_sweep(r, s, r->cfg.theta, false);
+}
+
+// n steps in a row: the observables of each but the last share a launch with the
+// reweight of the next.
+int enqueue_steps(pa_run* r, cudaStream_t s, int32_t n) {
+    for (int32_t i = 0; i < n; ++i) {
+        RunDev d = r->d;
+        CK(i == 0 ? pa::launch_tau(d, s) : pa::launch_obs_tau(d, r->cfg.theta, s));
+        if (r->cfg.resample == PA_RESAMPLE_MULTINOMIAL) CK(pa::launch_multinomial(d, s));
+        d.clear_hist = 1u;
+        CK(pa::launch_resample(d, s));
+        CK(pa::launch_sweep(r->d, r->cfg.theta, r->sweep_grid, s));
+    }
+    if (n > 0) CK(pa::launch_obs(r->d, r->cfg.theta, s));
+    return PA_OK;
 }
 
 }  // namespace
@@ -655,8 +670,7 @@ int pa_run_steps(pa_run* r, int32_t nsteps) {
     if (!r->graph && nsteps >= GRAPH_FROM) {
         if (!r->cap_stream) CK(cudaStreamCreateWithFlags(&r->cap_stream, cudaStreamNonBlocking));
         CK(cudaStreamBeginCapture(r->cap_stream, cudaStreamCaptureModeThreadLocal));
-        int rc = PA_OK;
-        for (int i = 0; i < GRAPH_STEPS && rc == PA_OK; ++i) rc = enqueue_step(r, r->cap_stream);
+        const int rc = enqueue_steps(r, r->cap_stream, GRAPH_STEPS);
         cudaGraph_t g = nullptr;
         const cudaError_t e = cudaStreamEndCapture(r->cap_stream, &g);
         if (rc || e != cudaSuccess || !g) {
@@ -673,13 +687,7 @@ int pa_run_steps(pa_run* r, int32_t nsteps) {
     int32_t i = 0;
     if (r->graph)
         for (; i + GRAPH_STEPS <= nsteps; i += GRAPH_STEPS) CK(cudaGraphLaunch(r->graph, r->stream));
-    // kernel timing covers pa_step's launches only
-    const bool prof = r->prof;
-    r->prof = false;
-    int rc = PA_OK;
-    for (; i < nsteps && rc == PA_OK; ++i) rc = enqueue_step(r, r->stream);
-    r->prof = prof;
-    return rc;
+    return enqueue_steps(r, r->stream, nsteps - i);  // kernel timing covers pa_step's launches only
 }
 
 int pa_status(pa_run* r) {

@@ -50,7 +50,13 @@ struct DevState {
     uint32_t over_n;              // copies left to k_spread: entries of RunDev::srcmap2
     uint32_t pad;
 };
-static_assert(sizeof(DevState) <= 256, "DevState must fit its slot");
+// Results of a reweight that shares its launch with the observables of the step
+// before, until the last block moves them to DevState (second half of its slot).
+struct TauNext {
+    double lnQ, lnZ, S;
+    uint32_t kref;
+};
+static_assert(sizeof(DevState) <= 128 && sizeof(TauNext) <= 128, "DevState's slot is 256 bytes");
 
 // Per-step record, same layout as pa_obs.
 static_assert(sizeof(pa_obs) == 104 && offsetof(pa_obs, sumM2) - offsetof(pa_obs, sumE) == 24 &&
@@ -189,7 +195,8 @@ __device__ __forceinline__ uint32_t pick(const uint4& v, uint32_t j) {
 // they touch memory, until all of its writes are visible.  Every block of every
 // kernel of the chain passes here first, so "the predecessor has finished" holds
 // for all earlier ones too.  A plain launch passes at once.  On GB300 a step of
-// 1000 replicas at L = 16 took 39.1 us by single launches and takes 31.3 us so.
+// 1000 replicas at L = 16 took 39.1 us by single launches and 31.3 us so, all else
+// equal.
 // Letting the successor in at the start of a kernel (launch_dependents) fills
 // SMs with waiting blocks that keep out the sweep's: up to 78 us instead of 34 for
 // 4099 spin glasses of L = 6.
@@ -291,6 +298,8 @@ cudaError_t launch_init(const RunDev& d, cudaStream_t s);
 cudaError_t launch_sweep(const RunDev& d, int nsweeps, int grid, cudaStream_t s);
 int sweep_grid(const RunDev& d);
 cudaError_t launch_tau(const RunDev& d, cudaStream_t s);
+// the observables of the step that has been swept, and the next step's reweight
+cudaError_t launch_obs_tau(const RunDev& d, int nsweeps, cudaStream_t s);
 cudaError_t launch_resample(const RunDev& d, cudaStream_t s);
 // Redistribution between virtual GPUs (pa_resample_begin / pa_resample_finish):
 // the counts and scan alone, then the gather into a permuted slot order.

@@ -113,6 +113,38 @@ __device__ __forceinline__ void split32(double x, uint32_t& n, uint32_t& F) {
 #define PA_TAU_CTAS 33
 #endif
 constexpr uint32_t TAU_CTAS = PA_TAU_CTAS;
+__device__ __forceinline__ TauNext* tau_next(const RunDev& d) {
+    return reinterpret_cast<TauNext*>(reinterpret_cast<uint8_t*>(d.st) + 128);
+}
+
+// The run's scalars after the reweight of step i, by one thread, once every block
+// has read the old ones.
+__device__ __forceinline__ void tau_advance(DevState* st, uint32_t i, uint32_t R, uint32_t cur,
+                                            uint32_t epoch, uint32_t kref) {
+    st->tau_done = 0;
+    st->kref = kref;
+    st->step = i;
+    st->R_prev = R;
+    st->epoch = epoch + 1;
+    st->tile_counter = 0;
+    st->over_n = 0;
+    st->src = cur;
+    st->cur = cur ^ 1u;
+    st->active = 1;
+}
+__device__ __forceinline__ void tau_advance_next(const RunDev& d, uint32_t i, uint32_t R, uint32_t cur,
+                                                 uint32_t epoch) {
+    const TauNext* nx = tau_next(d);
+    DevState* st = d.st;
+    st->lnQ = __ldcg(&nx->lnQ);
+    st->lnZ = __ldcg(&nx->lnZ);
+    st->S = __ldcg(&nx->S);
+    tau_advance(st, i, R, cur, epoch, __ldcg(&nx->kref));
+}
+
+// WITH_OBS: one more block of the launch takes the observables of the step
+// before, which read ln Q and ln Z: the new ones wait in TauNext.
+template <bool WITH_OBS>
 __device__ __forceinline__ bool tau_run(const RunDev& d, uint32_t blk, uint32_t nblk) {
     DevState* st = d.st;
     __shared__ double s_prod[TAU_HELD];
@@ -214,39 +246,37 @@ __device__ __forceinline__ bool tau_run(const RunDev& d, uint32_t blk, uint32_t 
             const long long Eref =
                 2 * (2 * (long long)kref + (long long)(negbonds & 1u)) - (long long)d.dim * d.N;
             const double lnQ = __dsub_rn(__dsub_rn(ln, lnR), __dmul_rn(db, (double)Eref));
-            st->lnQ = lnQ;
-            st->lnZ = __dadd_rn(lnZ, lnQ);
-            st->S = S;
+            if constexpr (WITH_OBS) {
+                *tau_next(d) = TauNext{lnQ, __dadd_rn(lnZ, lnQ), S, kref};
+            } else {
+                st->lnQ = lnQ;
+                st->lnZ = __dadd_rn(lnZ, lnQ);
+                st->S = S;
+            }
         }
     }
-    if (nblk > 1) {
+    const uint32_t arrivals = nblk + (WITH_OBS ? 1u : 0u);
+    if (arrivals > 1) {
         __shared__ bool s_last;
         __syncthreads();
         if (t == 0) {
             __threadfence();
-            s_last = atomicAdd(&st->tau_done, 1ull) == (unsigned long long)(nblk - 1);
+            s_last = atomicAdd(&st->tau_done, 1ull) == (unsigned long long)(arrivals - 1);
+            if (WITH_OBS) __threadfence();
         }
         __syncthreads();
         if (!s_last) return false;
     }
     if (t == 0) {
-        st->tau_done = 0;
-        st->kref = kref;
-        st->step = i;
-        st->R_prev = R;
-        st->epoch = epoch + 1;
-        st->tile_counter = 0;
-        st->over_n = 0;
-        st->src = cur;
-        st->cur = cur ^ 1u;
-        st->active = 1;
+        if constexpr (WITH_OBS) tau_advance_next(d, i, R, cur, epoch);
+        else tau_advance(st, i, R, cur, epoch, kref);
     }
     return true;
 }
 
 __global__ void __launch_bounds__(256) k_tau(__grid_constant__ const RunDev d) {
     chain_wait();
-    tau_run(d, blockIdx.x, gridDim.x);
+    tau_run<false>(d, blockIdx.x, gridDim.x);
 }
 
 // CTAs of a run's reweight: one per TAU_LEVELS levels, at most TAU_CTAS.
@@ -268,7 +298,7 @@ __global__ void __launch_bounds__(256) k_tau_batched(BatchDev b) {
     stage_run(&b.runs[blockIdx.x], s_d);
     __syncthreads();
     const RunDev& d = s_d;
-    if (!tau_run(d, blockIdx.y, nblk)) return;
+    if (!tau_run<false>(d, blockIdx.y, nblk)) return;
     __syncthreads();
     for (uint32_t k = threadIdx.x; k < (uint32_t)d.bins; k += blockDim.x) d.hist[k] = 0u;
     if (threadIdx.x < 2) d.accum[threadIdx.x] = 0ull;
@@ -926,6 +956,30 @@ __global__ void __launch_bounds__(256) k_obs(__grid_constant__ const RunDev d, i
     obs_run(d, nsweeps);
 }
 
+// The observables of the swept step (last block) beside the reweight of the
+// next (the others): neither waits for the other's result, and the chain of a
+// step in a run of steps is a kernel shorter.  us per step on GB300: 1000 replicas at
+// L = 16 22.9 -> 20.9, 4099 x 3D L = 6 31.1 -> 28.8, 20480 x L = 64 (theta = 1) 75.2 -> 72.8.
+__global__ void __launch_bounds__(256) k_obs_tau(__grid_constant__ const RunDev d, int nsweeps) {
+    chain_wait();
+    if (blockIdx.x + 1 < gridDim.x) {
+        tau_run<true>(d, blockIdx.x, gridDim.x - 1);
+        return;
+    }
+    DevState* st = d.st;
+    const uint32_t i = st->step + 1, R = st->R, cur = st->cur, epoch = st->epoch;
+    obs_run(d, nsweeps);
+    if (threadIdx.x >= 32) return;
+    __syncwarp();
+    if (threadIdx.x == 0 && i <= (uint32_t)d.K && R != 0) {
+        __threadfence();
+        if (atomicAdd(&st->tau_done, 1ull) == (unsigned long long)(gridDim.x - 1)) {
+            __threadfence();
+            tau_advance_next(d, i, R, cur, epoch);
+        }
+    }
+}
+
 __global__ void __launch_bounds__(256) k_obs_batched(BatchDev b) {
 #if PA_RS_STAGE
     __shared__ RunDev s_d;
@@ -944,6 +998,12 @@ cudaError_t launch_tau(const RunDev& d, cudaStream_t s) {
     RunDev dd = d;
     void* args[] = {&dd};
     return launch_chained((const void*)k_tau, dim3(tau_ctas(d.bins)), dim3(256), 0, s, args);
+}
+
+cudaError_t launch_obs_tau(const RunDev& d, int nsweeps, cudaStream_t s) {
+    RunDev dd = d;
+    void* args[] = {&dd, &nsweeps};
+    return launch_chained((const void*)k_obs_tau, dim3(tau_ctas(d.bins) + 1), dim3(256), 0, s, args);
 }
 
 // One wave of resident CTAs (capped by the number of tiles), looked up once
