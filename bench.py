@@ -255,7 +255,7 @@ def config1_measure(P, procs: int) -> dict:
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     torch.cuda.synchronize()
     e0.record(stream)
-    run.run_steps(CONFIG1["K"])  # one CUDA graph per step
+    run.run_steps(CONFIG1["K"])
     e1.record(stream)
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1)
@@ -961,7 +961,7 @@ def main():
         "plain": {"value": value_plain, "ms_per_step": ms_plain / args.steps,
                   "note": "one launch per kernel per step, kernel events on"},
         "batched": {"value": value, "ms_per_step": ms_graph / args.steps,
-                    "note": "one CUDA graph per step (pa_run_steps)"},
+                    "note": "pa_run_steps"},
         "kernels_ms_per_step": {k: (v[1] / max(v[0], 1)) for k, v in prof.items()},
         "sweep_attempts_per_ns_kernel": sweep_attempts_per_launch / (sweep_ms * 1e6),
         "roofline": {"bound": "alu", "achieved": achieved_tops, "peak": int_peak,

@@ -386,9 +386,10 @@ int pa_checkpoint(pa_run* run, void* host_dst, size_t bytes);
 int pa_restore(pa_run* run, const void* host_src, size_t bytes);
 
 /* Kernel timing (for benchmarks): while enabled, every kernel the run
- * enqueues outside a CUDA graph is bracketed by CUDA events on the run's
- * stream.  pa_profile_read synchronises and returns, per kernel kind
- * (0 reweight/tau, 1 resample: counts + scan + gather, 2 sweep, 3 observables),
+ * enqueues outside pa_run_steps is bracketed by CUDA events on the run's
+ * stream (which also keeps a step's kernels from overlapping at their ends).  pa_profile_read synchronises and returns, per kernel kind
+ * (0 reweight/tau, 1 resample: its draws, counts + scan + gather, 2 sweep, 3
+ * observables),
  * the number of launches and their summed device time in ms since the last
  * reset. */
 int pa_profile(pa_run* run, int32_t enable);
@@ -436,8 +437,10 @@ int pa_batch_profile_read(pa_batch* batch, int64_t* steps, double ms[4], int32_t
 /* Sweep classes and their launch shape: info = {layout, dim, L, model,
  * number of runs, warps per block, slots, slots per claim}.  The classes of
  * one step run as parallel branches.  pa_batch_set_shape chooses one class's
- * warps per block (2, 4 or 8; the L = 64 register kernel has 16 only; 0 keeps
- * the current value) and slots per claim (1, 2, 4, 8, 16 or 32; 0 picks the
+ * warps per block (2, 4 or 8; the register kernels have one shape only; 0 keeps
+ * the current value; the replica-sliced kernel's blocks are teams of a size that
+ * the lattice fixes, and 8 selects its form with four lanes per group of sites, 2
+ * and 4 the one with one lane) and slots per claim (1, 2, 4, 8, 16 or 32; 0 picks the
  * largest that leaves about four claims per resident warp).  Results do not
  * depend on the shape. */
 int pa_batch_num_classes(pa_batch* batch);

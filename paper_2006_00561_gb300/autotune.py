@@ -3,13 +3,14 @@
 For every sweep class of a batch (runs sharing layout, dim, L and model) it
 times whole batched steps with each candidate shape and keeps the fastest.  A
 shape is (warps per block, slots per claim):
-  * warps per block: 2, 4 or 8 (replicas in flight per CTA: one per warp for
-    the warp-per-replica kernels, 32 per warp for the replica-sliced one); the
-    L = 64 register kernel has a single block shape;
+  * warps per block: 2, 4 or 8; for the replica-sliced kernel 8 is its form
+    with four lanes per group of sites, 2 and 4 the one with one lane (its blocks
+    are teams of a size that the lattice fixes); the register kernels have a
+    single block shape;
   * slots per claim: how many consecutive replicas of one run a warp claims
     at a time from the class's slot space (1 .. 32, or 0 for the engine's
     automatic choice of about four claims per resident warp).  The
-    replica-sliced kernel (packed lattices with L <= 32) always claims 32.
+    replica-sliced kernel always claims 32.
 The launch shape never changes the results (random numbers are keyed by
 replica and site, not by thread), so the timed steps are real steps of the
 runs.  Choices are cached per (GPU, class, slot count rounded to a power of
@@ -35,7 +36,7 @@ def _key(gpu: str, c: dict) -> str:
 
 
 def replica_sliced(c: dict) -> bool:
-    """The class runs the replica-sliced kernel (32 replicas per warp, claims
+    """The class runs the replica-sliced kernel (32 replicas per block, claims
     of 32 slots): packed layout with L <= 32."""
     return c["layout"] == 1 and c["L"] <= 32
 
