@@ -148,7 +148,9 @@ __device__ __forceinline__ void load_unit(const uint8_t* src, bool i8, uint32_t 
             const int r = u * G::UROWS + q;
             uint4 b = make_uint4(0, 0, 0, 0);
             if (valid && r < G::RW) b = *reinterpret_cast<const uint4*>(src + 4 * (size_t)r);
-            row[q] = b.x, row[q + 1] = b.y, row[q + 2] = b.z, row[q + 3] = b.w;
+            // a loaded population may have bits set beyond the row: they are not spins
+            row[q] = b.x & G::ROWMASK, row[q + 1] = b.y & G::ROWMASK;
+            row[q + 2] = b.z & G::ROWMASK, row[q + 3] = b.w & G::ROWMASK;
         }
         if constexpr (L >= 32) {
 #pragma unroll
