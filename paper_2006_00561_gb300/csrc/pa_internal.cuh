@@ -197,6 +197,9 @@ __device__ __forceinline__ uint32_t pick(const uint4& v, uint32_t j) {
 // for all earlier ones too.  A plain launch passes at once.  On GB300 a step of
 // 1000 replicas at L = 16 took 39.1 us by single launches and 31.3 us so, all else
 // equal.
+// What the predecessors write is not read-only for such a kernel's lifetime, which
+// starts before the wait: its pointers carry no __restrict__, and it takes plain or
+// __ldcg loads, never __ldg (a compiler may move invariant loads above the wait).
 // Letting the successor in at the start of a kernel (launch_dependents) fills
 // SMs with waiting blocks that keep out the sweep's: up to 78 us instead of 34 for
 // 4099 spin glasses of L = 6.

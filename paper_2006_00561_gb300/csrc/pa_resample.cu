@@ -165,7 +165,7 @@ __device__ __forceinline__ bool tau_run(const RunDev& d, uint32_t blk, uint32_t 
         return blk == 0;
     }
     const double db = d.dbeta[i];
-    const double* __restrict__ D = d.dtab + (size_t)d.dsel[i] * bins;
+    const double* D = d.dtab + (size_t)d.dsel[i] * bins;
     // reference level: lowest occupied when cooling, highest when heating
     const bool heating = db < 0.0;
     if (t == 0) s_sum = 0;
@@ -429,9 +429,9 @@ __device__ __forceinline__ void spread_run(const RunDev& d, uint32_t blk, uint32
     for (uint32_t e = blk; e < n; e += nblk) {
         const uint32_t* at = d.srcmap2 + 3 * (size_t)e;
         const uint32_t rep = at[0], dst = at[1], copies = at[2];
-        const uint4* __restrict__ from = reinterpret_cast<const uint4*>(d.spins[src]) + (size_t)rep * CH;
-        uint4* __restrict__ to = reinterpret_cast<uint4*>(d.spins[src ^ 1u]) + (size_t)dst * CH;
-        for (uint32_t it = threadIdx.x; it < copies * CH; it += 256) __stcs(to + it, __ldg(from + it % CH));
+        const uint4* from = reinterpret_cast<const uint4*>(d.spins[src]) + (size_t)rep * CH;
+        uint4* to = reinterpret_cast<uint4*>(d.spins[src ^ 1u]) + (size_t)dst * CH;
+        for (uint32_t it = threadIdx.x; it < copies * CH; it += 256) __stcs(to + it, __ldcg(from + it % CH));
         const uint32_t level = d.ebin[src][rep];
         const int32_t mag = d.mag[src][rep];
         for (uint32_t k = threadIdx.x; k < copies; k += 256) {
@@ -621,9 +621,8 @@ __device__ __forceinline__ void resample_tile(const RunDev& d, uint32_t tile, ui
         // it / CH for it < RS_TILE * CH: the product with ceil(2^32 / CH) is exact
         // while it * CH < 2^32 (CH <= 1024)
         const uint32_t recip = CH > 1 ? 0xffffffffu / CH + 1u : 0u;
-        const uint4* __restrict__ srcp =
-            reinterpret_cast<const uint4*>(d.spins[src]) + (size_t)base * CH;
-        uint4* __restrict__ dstp = reinterpret_cast<uint4*>(d.spins[src ^ 1u]);
+        const uint4* srcp = reinterpret_cast<const uint4*>(d.spins[src]) + (size_t)base * CH;
+        uint4* dstp = reinterpret_cast<uint4*>(d.spins[src ^ 1u]);
         const uint32_t items = nsurv * CH;
         for (uint32_t it0 = t; it0 < items; it0 += RS_THREADS * GU) {
             uint4 v[GU];
@@ -632,7 +631,7 @@ __device__ __forceinline__ void resample_tile(const RunDev& d, uint32_t tile, ui
                 const uint32_t it = it0 + (uint32_t)u * RS_THREADS;
                 if (it < items) {
                     const uint32_t jl = recip ? __umulhi(it, recip) : it;
-                    v[u] = __ldg(srcp + (size_t)sm.surv[jl] * CH + (it - jl * CH));
+                    v[u] = __ldcg(srcp + (size_t)sm.surv[jl] * CH + (it - jl * CH));
                 }
             }
 #pragma unroll

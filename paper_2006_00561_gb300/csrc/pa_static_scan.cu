@@ -45,24 +45,23 @@ static __device__ __align__(256) StaticScanScratch g_scan_scratch;
 // replicas move as 16-byte words.
 template <bool VEC>
 __global__ void __launch_bounds__(SS_THREADS)
-    k_static_counts(StaticScanScratch* __restrict__ s, const uint32_t* __restrict__ ebin, uint32_t R,
-                    const uint32_t* __restrict__ tab_n, const uint32_t* __restrict__ tab_F,
-                    uint32_t bins, uint32_t step, uint32_t ctr3, uint32_t k0, uint32_t k1,
-                    uint32_t* __restrict__ counts) {
+    k_static_counts(StaticScanScratch* s, const uint32_t* ebin, uint32_t R, const uint32_t* tab_n,
+                    const uint32_t* tab_F, uint32_t bins, uint32_t step, uint32_t ctr3, uint32_t k0,
+                    uint32_t k1, uint32_t* counts) {
     __shared__ uint32_t s_warp[SS_THREADS / 32];
     chain_wait();
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const uint32_t base = blockIdx.x * SS_TILE;
-    uint32_t sum = 0;
+    uint32_t sum = 0, r[SS_ITEMS];
     bool bad = false;
 #pragma unroll
     for (int j0 = 0; j0 < SS_ITEMS; j0 += 4) {
         const uint32_t i0 = base + (uint32_t)t * SS_ITEMS + j0;
         uint4 u = make_uint4(0, 0, 0, 0);
-        uint32_t lev[4] = {0, 0, 0, 0}, r[4];
+        uint32_t lev[4] = {0, 0, 0, 0};
         if (i0 < R) u = philox(i0 >> 2, step, 0u, ctr3, k0, k1);
         if (VEC && i0 + 4 <= R) {
-            const uint4 e4 = __ldg(reinterpret_cast<const uint4*>(ebin + i0));
+            const uint4 e4 = *reinterpret_cast<const uint4*>(ebin + i0);
             lev[0] = e4.x, lev[1] = e4.y, lev[2] = e4.z, lev[3] = e4.w;
         } else {
 #pragma unroll
@@ -77,15 +76,19 @@ __global__ void __launch_bounds__(SS_THREADS)
                 if (k < bins) v = tab_n[k] + (pick(u, (uint32_t)j) < tab_F[k] ? 1u : 0u);
                 else bad = true;
             }
-            r[j] = v;
+            r[j0 + j] = v;
             sum += v;
         }
+    }
+#pragma unroll
+    for (int j0 = 0; j0 < SS_ITEMS; j0 += 4) {  // after all loads: the compiler may not move them up
+        const uint32_t i0 = base + (uint32_t)t * SS_ITEMS + j0;
         if (VEC && i0 + 4 <= R) {
-            *reinterpret_cast<uint4*>(counts + i0) = make_uint4(r[0], r[1], r[2], r[3]);
+            *reinterpret_cast<uint4*>(counts + i0) = make_uint4(r[j0], r[j0 + 1], r[j0 + 2], r[j0 + 3]);
         } else {
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                if (i0 + j < R) counts[i0 + j] = r[j];
+                if (i0 + j < R) counts[i0 + j] = r[j0 + j];
         }
     }
     sum = __reduce_add_sync(0xffffffffu, sum);
@@ -101,8 +104,8 @@ __global__ void __launch_bounds__(SS_THREADS)
 
 template <bool VEC>
 __global__ void __launch_bounds__(SS_THREADS)
-    k_static_offsets(const StaticScanScratch* __restrict__ s, const uint32_t* __restrict__ counts,
-                     uint32_t R, uint32_t* __restrict__ offsets, uint32_t* __restrict__ total) {
+    k_static_offsets(const StaticScanScratch* s, const uint32_t* counts, uint32_t R,
+                     uint32_t* offsets, uint32_t* total) {
     __shared__ uint32_t s_warp[SS_THREADS / 32], s_before[SS_THREADS / 32];
     chain_wait();
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
