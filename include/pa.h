@@ -267,10 +267,12 @@ int pa_bench_intops(int32_t kind, int32_t iters, void* out_dev, int64_t out_word
 #define PA_DEBUG_WITHHOLD_PREFIX 1u
 int pa_debug(pa_run* run, uint32_t flags);
 
-/* nsteps calls of pa_step.  Long calls (256 steps and more) and those after
- * them replay a CUDA graph of eight steps, which is captured on first use (on
- * a private stream, then launched on the run's stream); shorter ones enqueue the
- * kernels.  Same results as nsteps pa_step calls. */
+/* nsteps calls of pa_step, asynchronous however long the call and however many
+ * follow each other: what goes beyond a share of the stream's launch queue
+ * replays CUDA graphs of the steps, captured on first use (on a private stream,
+ * then launched on the run's stream); the rest, and every step while the run's
+ * stream is under capture, is enqueued kernel by kernel.  Same results as nsteps
+ * pa_step calls. */
 int pa_run_steps(pa_run* run, int32_t nsteps);
 
 /* Synchronises the run's stream and copies the observables of the latest

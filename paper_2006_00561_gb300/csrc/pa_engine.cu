@@ -33,7 +33,11 @@ struct pa_run {
     std::vector<double> dyn_table[2];  // host copies of the two dynamic weight slots
     DevState init_state;
     cudaStream_t cap_stream;
-    cudaGraphExec_t graph;
+    // pa_run_steps: GRAPH_STEPS steps that each begin with the observables of the one
+    // before, one whole step, and the kernels enqueued singly since the host last
+    // waited for the stream
+    cudaGraphExec_t graph, graph_one;
+    int64_t queued;
     size_t hist_bytes;  // accum (16 B) + histogram
     // kernel timing
     bool prof;
@@ -57,12 +61,10 @@ namespace {
 
 constexpr size_t ALIGN = 256;
 
-// Steps in the CUDA graph of pa_run_steps, and the steps of a call from which
-// one is built.  Chained launches run a step as fast as the graph does (31.8
-// against 31.7 us for 1000 replicas at L = 16 on GB300 when this was measured, 39 us
-// with a graph of one step), and the graph's construction and first launch cost
-// 100 us; a long call takes it to leave the host free (1.5 us a step instead of 7.5).
-constexpr int32_t GRAPH_STEPS = 8, GRAPH_FROM = 256;
+// pa_run_steps: the steps of its CUDA graph; the single launches that it leaves in
+// the stream's queue before it takes graphs; and the steps that it enqueues before it
+// builds one, while the device is busy with them.  See there.
+constexpr int32_t GRAPH_STEPS = 8, LAUNCH_BUDGET = 768, LEAD_STEPS = 32;
 
 size_t align_up(size_t v) { return (v + ALIGN - 1) / ALIGN * ALIGN; }
 
@@ -238,6 +240,7 @@ int sticky_to_code(uint32_t bits) {
 
 int read_state(pa_run* r, DevState* out) {
     CK(cudaStreamSynchronize(r->stream));
+    r->queued = 0;
     CK(cudaMemcpy(out, r->d.st, sizeof(DevState), cudaMemcpyDeviceToHost));
     return PA_OK;
 }
@@ -356,18 +359,44 @@ int enqueue_step(pa_run* r, cudaStream_t s) {
 }
 
 // n steps in a row: the observables of each but the last share a launch with the
-// reweight of the next.
-int enqueue_steps(pa_run* r, cudaStream_t s, int32_t n) {
-    for (int32_t i = 0; i < n; ++i) {
+// reweight of the next.  open: those of the step before the first are still to be
+// taken; close: those of the last are taken too.
+int enqueue_steps(pa_run* r, cudaStream_t s, int32_t n, bool open = false, bool close = true) {
+    for (int32_t i = 0; i < n; ++i, open = true) {
         RunDev d = r->d;
-        CK(i == 0 ? pa::launch_tau(d, s) : pa::launch_obs_tau(d, r->cfg.theta, s));
+        CK(open ? pa::launch_obs_tau(d, r->cfg.theta, s) : pa::launch_tau(d, s));
         if (r->cfg.resample == PA_RESAMPLE_MULTINOMIAL) CK(pa::launch_multinomial(d, s));
         d.clear_hist = 1u;
         CK(pa::launch_resample(d, s));
         CK(pa::launch_sweep(r->d, r->cfg.theta, r->sweep_grid, s));
     }
-    if (n > 0) CK(pa::launch_obs(r->d, r->cfg.theta, s));
+    if (open && close) CK(pa::launch_obs(r->d, r->cfg.theta, s));
     return PA_OK;
+}
+
+// Kernels of a step of enqueue_steps.
+int64_t step_launches(const pa_run* r) {
+    return 3 + (r->d.spread ? 1 : 0) + (r->cfg.resample == PA_RESAMPLE_POISSON ? 1 : 0) +
+           (r->cfg.resample == PA_RESAMPLE_MULTINOMIAL ? 3 : 0);
+}
+
+// The graph of n steps, captured on a private stream; false leaves *out empty.
+bool capture_steps(pa_run* r, int32_t n, bool open, bool close, cudaGraphExec_t* out) {
+    cudaGraph_t g = nullptr;
+    bool ok = r->cap_stream ||
+              cudaStreamCreateWithFlags(&r->cap_stream, cudaStreamNonBlocking) == cudaSuccess;
+    ok = ok && cudaStreamBeginCapture(r->cap_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+    if (ok) {
+        const int rc = enqueue_steps(r, r->cap_stream, n, open, close);
+        ok = cudaStreamEndCapture(r->cap_stream, &g) == cudaSuccess && rc == PA_OK && g;
+    }
+    ok = ok && cudaGraphInstantiate(out, g, 0) == cudaSuccess;
+    if (g) cudaGraphDestroy(g);
+    if (!ok) {
+        *out = nullptr;
+        (void)cudaGetLastError();  // the steps are then launched singly
+    }
+    return ok;
 }
 
 }  // namespace
@@ -426,7 +455,8 @@ int pa_init(const pa_config* cfg, void* ws, size_t bytes, void* stream, pa_run**
     r->dtab = dtab;
     r->ndist = (uint32_t)l.ndist;
     r->cap_stream = nullptr;
-    r->graph = nullptr;
+    r->graph = r->graph_one = nullptr;
+    r->queued = 0;
     r->ev_range = r->ev_copied = nullptr;
     r->prof = false;
     for (int k = 0; k < 4; ++k) {
@@ -665,29 +695,54 @@ int pa_debug(pa_run* r, uint32_t flags) {
     return PA_OK;
 }
 
+// The stream's queue holds 1024 launches; a call that finds it full waits until
+// the device has caught up.  So up to LAUNCH_BUDGET kernels are launched singly, and
+// what goes beyond them, or into a graph that is there already, goes by graphs, one
+// launch each: 200 multinomial steps of 65536 replicas at L = 64 (theta = 10, 314 ms on
+// GB300) return after 0.5 ms, singly after 44 ms, and 200 calls of one step after 1.3 ms
+// (83).  On the device a step takes as long either way (us, single / graph: 19.7 / 19.7
+// for 1000 replicas at L = 16, 27.9 / 27.8 for 4099 x 3D L = 6, 47.5 / 47.2 for 15001 by
+// multinomial draws; a graph of one step takes 1 us more).  But a graph's construction
+// and first launch take the host 100 us, which the steps enqueued ahead of it cover only
+// in part: with a budget of 128 launches, runs of 30 to 100 steps took 1 to 3 % longer.
 int pa_run_steps(pa_run* r, int32_t nsteps) {
     if (!r || nsteps < 0 || r->gather_pending) return PA_ERR_INVALID_ARG;
-    if (!r->graph && nsteps >= GRAPH_FROM) {
-        if (!r->cap_stream) CK(cudaStreamCreateWithFlags(&r->cap_stream, cudaStreamNonBlocking));
-        CK(cudaStreamBeginCapture(r->cap_stream, cudaStreamCaptureModeThreadLocal));
-        const int rc = enqueue_steps(r, r->cap_stream, GRAPH_STEPS);
-        cudaGraph_t g = nullptr;
-        const cudaError_t e = cudaStreamEndCapture(r->cap_stream, &g);
-        if (rc || e != cudaSuccess || !g) {
-            if (g) cudaGraphDestroy(g);
-            return rc ? rc : PA_ERR_CUDA;
-        }
-        const cudaError_t ie = cudaGraphInstantiate(&r->graph, g, 0);
-        cudaGraphDestroy(g);
-        if (ie != cudaSuccess) {
-            r->graph = nullptr;
-            return PA_ERR_CUDA;
-        }
+    if (nsteps == 0) return PA_OK;
+    const cudaStream_t s = r->stream;
+    const int64_t per = step_launches(r);
+    bool graphs = r->queued + nsteps * per + 1 > LAUNCH_BUDGET || (r->graph && nsteps > GRAPH_STEPS);
+    if (graphs) {  // a stream under capture queues nothing, and takes no graph
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        CK(cudaStreamIsCapturing(s, &cs));
+        graphs = cs == cudaStreamCaptureStatusNone;
     }
-    int32_t i = 0;
-    if (r->graph)
-        for (; i + GRAPH_STEPS <= nsteps; i += GRAPH_STEPS) CK(cudaGraphLaunch(r->graph, r->stream));
-    return enqueue_steps(r, r->stream, nsteps - i);  // kernel timing covers pa_step's launches only
+    if (!graphs) {
+        r->queued += nsteps * per + 1;
+        return enqueue_steps(r, s, nsteps);
+    }
+    int32_t left = nsteps;
+    bool open = false;
+    if (left > GRAPH_STEPS) {
+        int32_t lead = 1;
+        if (!r->graph && r->queued < LEAD_STEPS * per)
+            lead = left - GRAPH_STEPS < LEAD_STEPS ? left - GRAPH_STEPS : LEAD_STEPS;
+        const int rc = enqueue_steps(r, s, lead, false, false);
+        if (rc) return rc;
+        r->queued += lead * per;
+        left -= lead;
+        open = true;
+        if (r->graph || capture_steps(r, GRAPH_STEPS, true, false, &r->graph))
+            for (; left >= GRAPH_STEPS; left -= GRAPH_STEPS) CK(cudaGraphLaunch(r->graph, s));
+    }
+    const bool one = left > 0 && left < GRAPH_STEPS && r->queued + left * per > LAUNCH_BUDGET &&
+                     (r->graph_one || capture_steps(r, 1, false, true, &r->graph_one));
+    if (!one) {
+        r->queued += left * per + 1;
+        return enqueue_steps(r, s, left, open);
+    }
+    if (open) CK(pa::launch_obs(r->d, r->cfg.theta, s));
+    for (; left > 0; --left) CK(cudaGraphLaunch(r->graph_one, s));
+    return PA_OK;
 }
 
 int pa_status(pa_run* r) {
@@ -1156,6 +1211,7 @@ void pa_free(pa_run* r) {
     if (r->ev_range) cudaEventDestroy(r->ev_range);
     if (r->ev_copied) cudaEventDestroy(r->ev_copied);
     if (r->graph) cudaGraphExecDestroy(r->graph);
+    if (r->graph_one) cudaGraphExecDestroy(r->graph_one);
     if (r->cap_stream) cudaStreamDestroy(r->cap_stream);
     delete r;
 }
