@@ -13,8 +13,8 @@ shape is (warps per block, slots per claim):
     replica-sliced kernel always claims 32.
 The launch shape never changes the results (random numbers are keyed by
 replica and site, not by thread), so the timed steps are real steps of the
-runs.  Choices are cached per (GPU, class, slot count rounded to a power of
-two) in a JSON file.
+runs.  Choices are cached per (GPU, meaning of the shapes, class, slot count
+rounded to a power of two) in a JSON file.
 
 The resample's copy tile (replicas per tile, loads in flight per thread) sizes
 each run's lookback descriptors in its workspace, so it is fixed when the
@@ -26,27 +26,37 @@ import json
 import os
 
 WARPS = (2, 4, 8)
+SLICED = ((4, 0), (8, 0))  # the replica-sliced kernel's two forms: one lane, four lanes
 CHUNKS = (0, 4, 8, 16, 32)
 DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "pa_gb300", "autotune.json")
 
 
+# What a shape selects: to be raised when a kernel's shapes change their meaning,
+# so that a choice saved for the earlier kernel is not taken for this one.  2: the
+# replica-sliced kernel's blocks are teams and 8 is its form with four lanes; before,
+# 2, 4 and 8 were warps of 32 replicas each (saved without a number).
+SHAPES = 2
+
+
 def _key(gpu: str, c: dict) -> str:
     slots = 1 << max(0, int(c["slots"]) - 1).bit_length()
-    return f"{gpu}|layout{c['layout']}|d{c['dim']}|L{c['L']}|m{c['model']}|slots{slots}"
+    return f"{gpu}|shapes{SHAPES}|layout{c['layout']}|d{c['dim']}|L{c['L']}|m{c['model']}|slots{slots}"
 
 
 def replica_sliced(c: dict) -> bool:
     """The class runs the replica-sliced kernel (32 replicas per block, claims
-    of 32 slots): packed layout with L <= 32."""
-    return c["layout"] == 1 and c["L"] <= 32
+    of 32 slots): as pa.Batch.classes names it; of a class without a name, packed
+    layout with L <= 32."""
+    return c["kernel"] == "sliced" if "kernel" in c else c["layout"] == 1 and c["L"] <= 32
 
 
 def candidates(c: dict) -> list:
-    """(warps, chunk) shapes to try for one class."""
+    """(warps, chunk) shapes to try for one class: those that differ for the kernel
+    that it names, all that its layout may take without a name."""
     if c["layout"] == 1 and c["dim"] == 2 and c["L"] in (64, 128):
         return [(c["warps"], ch) for ch in CHUNKS]  # register kernels: one block shape
     if replica_sliced(c):
-        return [(w, 0) for w in WARPS]
+        return list(SLICED) if "kernel" in c else [(w, 0) for w in WARPS]
     return [(w, ch) for w in WARPS for ch in CHUNKS]
 
 

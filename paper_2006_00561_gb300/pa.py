@@ -536,8 +536,10 @@ class Batch:
         for c in range(int(lib().pa_batch_num_classes(C.c_void_p(self.h)))):
             info = (C.c_int32 * 8)()
             _check(lib().pa_batch_class_info(C.c_void_p(self.h), c, info), "pa_batch_class_info")
-            out.append(dict(zip(("layout", "dim", "L", "model", "runs", "warps", "slots",
-                                 "chunk"), list(info))))
+            k = dict(zip(("layout", "dim", "L", "model", "runs", "warps", "slots", "chunk"),
+                         list(info)))
+            register = k["layout"] == LAYOUT_PACKED and k["dim"] == 2 and k["L"] in (64, 128)
+            out.append(dict(k, kernel="register" if register else "sliced"))
         return out
 
     def profile(self, enable: bool):
