@@ -9,7 +9,7 @@ population buffers, far above the 129 MB L2), beta 0 -> 1 in 400 steps.
 The timed steps are steps W+1 .. W+K of that schedule.
 
 value     = spin-flip attempts per ns over the whole step (device time, CUDA
-            events on the run's stream, graph-replayed steps).
+            events on the run's stream, pa_run_steps).
 e2e       = the same metric through the C ABI with host buffers: every step
             uploads the population from pinned host memory (pa_load), steps
             with the new population copied back to that memory range by range
@@ -52,9 +52,9 @@ OPS_PER_ATTEMPT = 19.5
 ALU_PEAK_TOPS = 152 * 128 * 2.070e9 / 1e12
 # DRAM bytes of one sweep launch, from the ncu capture of the same kernel at
 # 2^20 replicas, four times L2 (profiles/k_sweep_l64_ising2d_L64_R2p18.md:
-# 538.5 MB read + 483.2 MB written), scaled by the replica count to 2^21.
+# 538.2 MB read + 483.2 MB written), scaled by the replica count to 2^21.
 # None whenever the kernel changes, until the next capture.
-SWEEP_TRAFFIC_BYTES_2P21 = (538.521344e6 + 483.193344e6) * 2
+SWEEP_TRAFFIC_BYTES_2P21 = (538.198272e6 + 483.17952e6) * 2
 # Slot ranges of the e2e step: each range's copy to the host (~0.7 ms at 1/8 of
 # 1 GiB) runs while the next range sweeps (~7 ms).
 E2E_CHUNKS = 8
@@ -244,8 +244,8 @@ def _config1_oracle(seed):
 
 
 def config1_measure(P, procs: int) -> dict:
-    """Config 1 in full: the whole run on the GPU (int8 layout, graph-replayed
-    steps, device time) and on the oracle, one process and one per host core
+    """Config 1 in full: the whole run on the GPU (int8 layout, one call of
+    pa_run_steps, device time) and on the oracle, one process and one per host core
     (different seeds; the seed-1 process is the GPU run's twin)."""
     import multiprocessing as mp
 
@@ -276,7 +276,7 @@ def config1_measure(P, procs: int) -> dict:
 
 def config2_measure(P) -> dict:
     """Config 2 in full: 2D Ising L = 64 packed, R0 = 2^17, beta 0 -> 1 in 200
-    steps, theta = 10, seed 2, every step graph-replayed; device time of the
+    steps, theta = 10, seed 2, one call of pa_run_steps; device time of the
     whole run (the paper's task at 6.4 times its per-GPU replica count)."""
     import torch
     stream = torch.cuda.Stream()
@@ -515,7 +515,7 @@ def serving_measure(P, prefix: int = 24) -> dict:
 def next_items_measure(P, steps: int = 5, R0: int = WORKLOAD["R0"]) -> dict:
     """The extensions of the fixed-schedule path, each on the headline workload
     (2D Ising L = 64 packed, theta = 10, beta 0 -> 1 in 400 steps):
-      poisson    -- Poisson copy counts (Sec. 2's draw): graph-replayed step rate
+      poisson    -- Poisson copy counts (Sec. 2's draw): step rate of pa_run_steps
                     and resample time per step (kernel events);
       multinomial -- the same for multinomial resampling (cumulative-weight scan,
                     R0 draws, then the scan and gather);
@@ -782,11 +782,11 @@ def main():
         if dist is not None:
             dist.barrier()
 
-    # warm-up (also captures the graph of one step)
+    # warm-up
     run.run_steps(args.warmup)
     run.observables()
 
-    # ---- timed region 1: graph-replayed steps (the headline) --------------
+    # ---- timed region 1: pa_run_steps (the headline) ----------------------
     first = run.state()["step"] + 1
     barrier()
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -990,9 +990,9 @@ def main():
                               "bytes_per_launch": res_bytes,
                               "sources_per_launch": sources, "R_in": R_in, "R_out": R_out,
                               "peak_note": "MEASURED_PEAKS.json hbm_gbs (of measured)"},
-        # kernels inside the headline timed region: k_tau, k_resample, the sweep
-        # kernel and k_obs per graph-replayed step
-        "gpu_launches": 4 * args.steps,
+        # kernels inside the headline timed region: k_tau, or k_obs_tau from the
+        # second step on, k_resample and the sweep kernel per step, then k_obs
+        "gpu_launches": 3 * args.steps + 1,
         "clocks": clk.result,
     }
     if e2e:
