@@ -8,13 +8,20 @@
 //              (Eq. 3) and the per-level weights tau_k = R0 D[|k - kref|] / S
 //              (Eq. 4, renormalised to R0), kept as n_k = floor(tau_k),
 //              F_k = floor(frac(tau_k) 2^32).
+//  k_poisson_counts, k_mn_tile_sums, k_mn_cum, k_mn_draw
+//              the copy counts of the Poisson and multinomial rules, ahead of the
+//              scan.
 //  k_resample  one pass over the population, one tile of RS_TILE replicas per
 //              CTA (or per group of CTAs that share its gather): copy counts r_j = n_k + [u_j < F_k] (nearest-integer rule),
 //              a single-pass exclusive scan with decoupled lookback across
 //              tiles, and the gather of r_j exact copies of replica j into slots
 //              o_j .. o_j + r_j - 1 of the other population buffer.
+//  k_spread    in runs whose beta steps leave replicas with many copies: the
+//              copies that k_resample's CTAs have left, shared out to all CTAs.
 //  k_obs       one CTA: exact integer sums over the histogram and the
 //              magnetisation accumulators, then the FP64 averages.
+//  k_obs_tau   in a row of steps: k_obs of a step beside k_tau of the next.
+//  k_gather, k_remap  the copies in the slot order of a redistribution.
 //
 // Floating point: IEEE double with explicit _rn intrinsics (no contraction),
 // summed in a fixed order, so the tables are the same bits as any other
@@ -107,8 +114,8 @@ __device__ __forceinline__ void split32(double x, uint32_t& n, uint32_t& F) {
         F = (uint32_t)(m >> (20 - e));
     }
 }
-// CTAs of a run at most: 33, 65 and 130 run alike on GB300 (14.7 us at 4097
-// levels, 24 us at 16385, timed by events around the launch).
+// CTAs of a run at most: 33, 65 and 130 ran alike on GB300 (14.7 us at 4097
+// levels, 24 us at 16385, before the products were formed by all threads).
 #ifndef PA_TAU_CTAS
 #define PA_TAU_CTAS 33
 #endif
@@ -325,7 +332,6 @@ struct ResampleSmem {
 #define PA_RS_GU 4
 #endif
 
-// Counts, scan and gather of tile `tile` of one run (all threads of the CTA).
 // Poisson(tau_k) copy count of replica i (Sec. 2), tau_k = n + F / 2^32: the
 // event count of a unit-rate Poisson process on [0, tau_k].  The fractional
 // interval contributes a Poisson(1) count thinned with keep probability
@@ -456,11 +462,12 @@ __global__ void __launch_bounds__(256) k_spread_batched(BatchDev b) {
 // HBM-bound default path); 2 takes the counts that the Poisson or multinomial
 // draws have left in d.counts; 3 chooses between the two per run (batches).
 //
-// SPLIT = false: the tile also gathers its replicas' spins (the batched form).
+// Counts, scan and gather of tile `tile` of one run (all threads of the CTA), or
+// its slice of them.  SPLIT = false: the tile also gathers its replicas' spins.
 // SPLIT = true: the tile writes, for each slot it fills, the index of the
 // source replica (srcmap) with the copied energy level and magnetisation, and
 // k_gather copies the spins afterwards over the whole new population (the
-// plain form).
+// redistribution's form).  SPREAD: copies beyond SPREAD_FROM are left to k_spread.
 template <int RULE, bool SPLIT, bool SPREAD>
 __device__ __forceinline__ void resample_tile(const RunDev& d, uint32_t tile, uint32_t slice,
                                               ResampleSmem& sm) {
@@ -1026,10 +1033,9 @@ static int resample_wave(const void* fn, int which, uint32_t tiles) {
 // PA_RS_SPLIT = 1: the plain resample is two kernels, counts + scan (with the
 // slot -> source map, levels and magnetisations) and then k_gather over the
 // whole new population; 0 (the default): one kernel that gathers tile by
-// tile (its figures here are from before its gather kept only data in
-// registers).  Measured on GB300 at 2^21 replicas, L = 64, same bits: one kernel
-// 0.366 ms with 4 loads in flight per thread in its gather (0.361 ms with 6,
-// the default); two kernels 0.374 ms (16 loads in flight per thread, 2 CTAs of
+// tile.  Measured on GB300 at 2^21 replicas, L = 64, same bits, before that gather
+// kept only data in registers (0.346 ms since): one kernel 0.366 ms with 4 loads in
+// flight per thread (0.361 ms with 6); two kernels 0.374 ms (16 loads in flight per thread, 2 CTAs of
 // 256 per SM), 0.380 ms (4 loads, 4 CTAs), 0.385 ms (8 loads, 3 CTAs).  The split
 // form serves the redistribution's gather (pa_resample_finish), whose slot
 // order is only known after the host has read the scan.

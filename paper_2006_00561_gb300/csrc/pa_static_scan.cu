@@ -37,7 +37,7 @@ static __device__ __align__(256) StaticScanScratch g_scan_scratch;
 // lookback saves re-reading the counts, but its prefix moves from tile to
 // tile in L2 round trips: 3 000 017 replicas (1465 tiles) took 64.4 us on GB300
 // with one descriptor at a time, 51.2 us with 32, 42.6 us with 256; the two passes
-// take 12.4 us a call (2.9 TB/s over the caller's arrays), 16.4 as single launches
+// take 12.6 us a call (2.9 TB/s over the caller's arrays), 16.4 as single launches
 // instead of a chain; up to 10^6 replicas a call is 6.1 to 6.6 us (8.2 to 12.3), its
 // launches and each pass's two dependent L2 round trips.
 //

@@ -2,8 +2,8 @@
 // L = 64, the workload of the paper's tests (Sec. 3 and 4), bit-packed one
 // 64-site row per 64-bit word.
 //
-// Same update rule and random numbers as the generic kernels of pa_sweep.cu
-// (checkerboard order, dE = 4 (2 - c_u), u = word h & 3 of the Philox block
+// Same update rule and random numbers as the replica-sliced kernel (pa_sliced.cuh:
+// checkerboard order, dE = 4 (2 - c_u), u = word h & 3 of the Philox block
 // with counter (2 g + colour, h >> 2, SWEEP | instance, slot), h = s >> 1, accept iff
 // dE <= 0 or u < T(beta_i, dE)), mapped for throughput:
 //   * one warp holds one replica for all theta sweeps, entirely in registers:
@@ -25,7 +25,7 @@
 //     the block index and the half-sweep, once per CTA into shared-memory
 //     tables: a block costs 14 of Philox's 20 multiplies.
 // Grid-stride (persistent) over replicas; the population size is read from
-// device memory.  The measurement epilogue is the one of the generic kernel.
+// device memory.  The measurement is fused, as in the replica-sliced kernel.
 #include "pa_internal.cuh"
 
 #include <cmath>
