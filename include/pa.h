@@ -342,7 +342,8 @@ int64_t pa_num_bins(int32_t dim, int32_t L);
 
 /* Replaces the current population with `count` replicas read from host memory
  * (what = PA_DUMP_SPINS: int8 +-1 per site in site order; PA_DUMP_SPINS_RAW:
- * the device layout, `stride` bytes per replica as pa_dump gives it), then
+ * the device layout, `stride` bytes per replica as pa_dump gives it; bits of a
+ * packed row word beyond the row are not spins), then
  * measures it (energy levels, magnetisations, histogram, observables record
  * of the current step) exactly as pa_sweep(run, 0) does.  count must lie in
  * 1 .. capacity; bytes >= count * (N or stride).  The step index, ln Z and
